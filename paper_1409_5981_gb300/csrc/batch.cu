@@ -9,7 +9,6 @@
 #include <algorithm>
 #include <vector>
 
-#include "binning.cuh"
 #include "internal.cuh"
 #include "m2l_table.cuh"
 
@@ -18,27 +17,6 @@ namespace pmmm {
 namespace {
 
 constexpr double kPi = 3.14159265358979323846;
-
-// system of particle i: offsets[s] <= i < offsets[s+1]
-__device__ __forceinline__ int system_of(const int64_t* __restrict__ off, int nsys, int64_t i) {
-  int lo = 0, hi = nsys;  // invariant: off[lo] <= i < off[hi]
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (off[mid] <= i) lo = mid;
-    else hi = mid;
-  }
-  return lo;
-}
-
-template <typename T>
-__global__ void bin_batched_kernel(const T* __restrict__ pos, const T* __restrict__ q, int64_t n,
-                                   const int64_t* __restrict__ offsets, int nsys, Geo g, int64_t Ksys,
-                                   uint32_t* __restrict__ keys, T* __restrict__ rec, int* __restrict__ err) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int s = system_of(offsets, nsys, i);
-  bin_record<T>(pos, q, i, g, (uint32_t)((int64_t)s * Ksys), keys, rec, err);
-}
 
 // Batched M2L on wavevector-major spectra ([k][c][system]): block = KT
 // consecutive wavevectors x BT systems.  Shared memory:
@@ -255,21 +233,6 @@ std::vector<int> build_m2l_table_int4(int p) {
     out[4 * i + 3] = t[i].s2;
   }
   return out;
-}
-
-cudaError_t launch_bin_batched(const void* pos, const void* q, bool fp64, int64_t n, const int64_t* offsets, int nsys,
-                               const Geo& g, int64_t Ksys, uint32_t* keys, void* rec, int* err, cudaStream_t s,
-                               int* nl) {
-  if (n <= 0) return cudaSuccess;
-  const unsigned blocks = (unsigned)((n + 255) / 256);
-  if (fp64)
-    bin_batched_kernel<double><<<blocks, 256, 0, s>>>((const double*)pos, (const double*)q, n, offsets, nsys, g, Ksys,
-                                                      keys, (double*)rec, err);
-  else
-    bin_batched_kernel<float><<<blocks, 256, 0, s>>>((const float*)pos, (const float*)q, n, offsets, nsys, g, Ksys,
-                                                     keys, (float*)rec, err);
-  ++*nl;
-  return cudaGetLastError();
 }
 
 cudaError_t launch_transpose(bool fp64, const void* in, void* out, int64_t R, int64_t Kh, cudaStream_t s, int* nl) {

@@ -72,11 +72,11 @@ __device__ __forceinline__ bool bin_axis_fast(float x, const Geo& g, int a, int*
   return true;
 }
 
-// Bins particle i: writes its key key0 + cell id and its record (u_x, u_y, u_z, q)
+// Bins particle i: writes and returns its key key0 + cell id and writes its record (u_x, u_y, u_z, q)
 // in input order, u being the position relative to the cell centre in units of
 // hs, rounded to T.  FP32 inputs take the fast path where it is exact.
 template <typename T>
-__device__ __forceinline__ void bin_record(const T* __restrict__ pos, const T* __restrict__ q, int64_t i,
+__device__ __forceinline__ uint32_t bin_record(const T* __restrict__ pos, const T* __restrict__ q, int64_t i,
                                            const Geo& g, uint32_t key0, uint32_t* __restrict__ keys,
                                            T* __restrict__ rec, int* __restrict__ err) {
   int ix[3];
@@ -103,7 +103,8 @@ __device__ __forceinline__ void bin_record(const T* __restrict__ pos, const T* _
       u[a] = (T)(rel * g.ihs);
     }
   }
-  keys[i] = key0 + (uint32_t)(ix[0] + g.n[0] * (ix[1] + g.n[1] * ix[2]));
+  const uint32_t key = key0 + (uint32_t)(ix[0] + g.n[0] * (ix[1] + g.n[1] * ix[2]));
+  keys[i] = key;
   using V = typename std::conditional<sizeof(T) == 4, float4, double4>::type;
   V o;
   o.x = u[0];
@@ -111,6 +112,7 @@ __device__ __forceinline__ void bin_record(const T* __restrict__ pos, const T* _
   o.z = u[2];
   o.w = q[i];
   reinterpret_cast<V*>(rec)[i] = o;
+  return key;
 }
 
 }  // namespace pmmm

@@ -77,16 +77,48 @@ enum ErrBits { ERRBIT_OUT_OF_BOX = 1, ERRBIT_NONFINITE = 2, ERRBIT_TIMEOUT = 4 }
 // Device error flag helpers
 __device__ __forceinline__ void set_err(int* err, int bit) { atomicOr(err, bit); }
 
+// ---------------------------------------------------------------- cellsort.cu
+// Work lists of an evaluation, built with the sort: exclusive sums over the cells
+// (K + 1 entries each, the last one the total).
+constexpr int PP_CHUNK = 32;  // target particles per near-field work item
+struct CellLists {
+  int* cs = nullptr;               // first sorted slot of each cell
+  uint32_t* cs_local = nullptr;    // scratch: the same within blocks of cells
+  uint32_t* item_start = nullptr;  // near-field work items
+  uint32_t* pair_start = nullptr;  // source pairs of the FP32 near field (FP64: null)
+  uint32_t* tot = nullptr;         // scratch, cell_list_totals(K) entries
+  unsigned int* ticket = nullptr;  // one zeroed counter, left zeroed
+  unsigned int* counter = nullptr;  // work counter of the near field, reset here
+};
+int64_t cell_list_totals(int64_t K);
+// Bins the particles (FP64 formula, binning.cuh): keys, records (u, q) in input order,
+// and the arrival number of every particle in its cell (count: K zeroed counters).
+// offsets (may be null: one system): particles offsets[s] ... offsets[s + 1] - 1 belong
+// to system s, whose cells are s * Ksys ... (device array of nsys + 1 entries).
+cudaError_t launch_bin_count(const void* pos, const void* q, bool fp64, int64_t n, const int64_t* offsets, int nsys,
+                             const Geo& g, int64_t Ksys, uint32_t* keys, uint32_t* arrival, uint32_t* count, void* rec,
+                             int* err, cudaStream_t s, int* nlaunch);
+// Stable sort by cell with the lists: vals (original index of each sorted slot),
+// keys_sorted (its cell), part[s] = rec[vals[s]] (position relative to the cell centre
+// in units of hs, and the charge), item_cell (the cell of every work item), src2 (FP32:
+// the pair-interleaved sources, 32 bytes per pair, layout in pp.cu) and zeroed energy
+// partials of the unused item slots (of all of them with zero_all: the per-target near
+// field accumulates into them).  count is left zeroed; order: scratch of n + 4 entries,
+// 16-byte aligned.
+cudaError_t launch_cell_sort(const uint32_t* keys, const uint32_t* arrival, uint32_t* count, const void* rec, bool fp64,
+                             int64_t n, int64_t K, const CellLists& l, uint32_t* order, uint32_t* vals,
+                             uint32_t* keys_sorted, void* part, void* src2, uint32_t* item_cell, double* epart,
+                             int64_t max_items, bool zero_all, cudaStream_t s, int* nlaunch);
+
 // ---------------------------------------------------------------- sort.cu
+// The radix sort of the allocation-free entry point (static_sort.cu), whose scratch
+// cannot hold a counter per cell.
 struct SortWork {
   uint32_t *keys0, *keys1, *vals0, *vals1;
   uint32_t* hist;    // [256 * ntiles_max]
   uint32_t* chunks;  // [scan chunk sums]
   int64_t cap;
 };
-int sort_tiles(int64_t n);
-size_t sort_hist_entries(int64_t n);
-size_t sort_chunk_entries(int64_t n);
 // Bins the particles (FP64 formula) and writes their records (u, q) in input order.
 cudaError_t launch_bin(const void* pos, const void* q, bool fp64, int64_t n, const Geo& g, uint32_t* keys, void* rec,
                        int* err, cudaStream_t s, int* nlaunch);
@@ -95,9 +127,6 @@ cudaError_t launch_radix_sort(SortWork& w, int64_t n, int key_bits, uint32_t** k
                               cudaStream_t s, int* nlaunch);
 cudaError_t launch_cell_bounds(const uint32_t* keys, int64_t n, int64_t K, int* cell_start, cudaStream_t s,
                                int* nlaunch);
-// In-place exclusive scan of n uint32 values (chunks: scratch of scan_chunk_count(n)).
-int64_t scan_chunk_count(int64_t n);
-cudaError_t launch_exclusive_scan(uint32_t* data, int64_t n, uint32_t* chunks, cudaStream_t s, int* nlaunch);
 
 // ---------------------------------------------------------------- p2m_l2p.cu
 // sparse (FP32, p <= 8): one thread per cell, crowded cells taken by the whole warp
@@ -202,9 +231,6 @@ cudaError_t launch_m2l_systems(int p, bool fp64, const void* Mt, const void* Gt,
 // Many systems on one plan: system s owns cells s*Ksys ... s*Ksys + Ksys - 1 of
 // a mesh of nsys*Ksys cells; the particles of system s are offsets[s] ...
 // offsets[s+1]-1 (device array of nsys+1 entries).
-cudaError_t launch_bin_batched(const void* pos, const void* q, bool fp64, int64_t n, const int64_t* offsets, int nsys,
-                               const Geo& g, int64_t Ksys, uint32_t* keys, void* rec, int* err, cudaStream_t s,
-                               int* nlaunch);
 // Entry table of the real-matrix M2L as 4 ints per entry (i1, s1, i2, s2), C*C entries.
 std::vector<int> build_m2l_table_int4(int p);
 // out[k][r] = in[r][k] for complex R x Kh (channel-major <-> wavevector-major spectra)
@@ -307,21 +333,6 @@ struct PPParams {
 // (n + K) / 2 + 1.
 int64_t pp_items_max(int64_t K, int64_t n);
 int64_t pp_pairs_max(int64_t K, int64_t n);
-// Near-field work lists: item_start / pair_start (exclusive scans of the per-cell
-// item and source-pair counts, K + 1 entries; pair_start may be null) and the
-// reset of the work counter; chunks: scratch of pp_lists_chunk_entries(K) entries.
-int64_t pp_lists_chunk_entries(int64_t K);
-cudaError_t launch_pp_lists(const int* cell_start, int64_t K, uint32_t* item_start, uint32_t* pair_start,
-                            uint32_t* chunks, unsigned int* counter, cudaStream_t s, int* nlaunch);
-// Sorted records part[s] = rec[vals[s]] (position relative to the cell centre in
-// units of hs, and the charge), the cell of every work item (item_cell), the FP32
-// pair-interleaved sources (src2 not null; 32 bytes per pair, layout in pp.cu) and
-// zeroed energy partials of the unused item slots (of all of them with zero_all:
-// the per-target kernel accumulates into them).
-cudaError_t launch_gather_lists(const void* rec, bool fp64, const uint32_t* vals, const uint32_t* keys,
-                                const int* cell_start, const uint32_t* item_start, const uint32_t* pair_start,
-                                int64_t n, int64_t K, void* part, void* src2, uint32_t* item_cell, double* epart,
-                                int64_t max_items, bool zero_all, cudaStream_t s, int* nlaunch);
 // Near field over the (2c+1)^3 cells plus the far field from `far`, written in
 // the caller's order to phi / force; energy and force partials per work item
 // (epart[max_items][4]).  Persistent warps fetch items from *counter.  With

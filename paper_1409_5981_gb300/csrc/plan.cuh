@@ -23,7 +23,6 @@ struct FarHook {
 struct pmmm_plan {
   using Dims = pmmm::Dims;
   using Geo = pmmm::Geo;
-  using SortWork = pmmm::SortWork;
   pmmm_config cfg;
   cudaStream_t stream = nullptr;
   int p = 0, C = 0, CG = 0;
@@ -44,10 +43,12 @@ struct pmmm_plan {
   int bchunks = 0;
   double* epart = nullptr;    // [max items][4]
   uint32_t* item_start = nullptr;  // [K+1] near-field work items per cell (scanned)
-  uint32_t* item_chunks = nullptr; // scan scratch
+  uint32_t* cell_count = nullptr;  // [K] particles per cell while sorting, zero between evaluations
+  uint32_t* cs_local = nullptr;    // [K+1] scan scratch
+  uint32_t* scan_tot = nullptr;    // block totals of the cell scan
   uint32_t* item_cell = nullptr;   // [max items]
   int64_t max_items = 0;
-  unsigned int* counter = nullptr; // near-field work counter
+  unsigned int* counter = nullptr; // near-field work counter, ticket of the cell scan
   uint32_t* pair_start = nullptr;  // [K+1] FP32 near-field source pairs per cell (scanned)
   void* src2 = nullptr;            // pair-interleaved FP32 sources
   int num_sms = 0;
@@ -97,14 +98,15 @@ struct pmmm_plan {
   void* hum = nullptr;                        // L2L child matrices, r^3 * C * C (or none)
   // particle workspace
   int64_t cap = 0;
-  SortWork sw{};
+  // keys by input order and sorted; arrival numbers, then original indices of the
+  // sorted slots; the arrival order
+  uint32_t *keys = nullptr, *keys_sorted = nullptr, *vals_sorted = nullptr, *order = nullptr;
   void *part = nullptr, *far = nullptr;
   // staging for pmmm_compute_host
   int64_t hcap = 0;
   void *hpos = nullptr, *hq = nullptr, *hphi = nullptr, *hforce = nullptr;
   // last evaluation
   int64_t n_last = 0;
-  uint32_t *keys_sorted = nullptr, *vals_sorted = nullptr;
   int launches = 0;
   size_t ws_bytes = 0;
   bool timing = false, timed = false;

@@ -56,13 +56,10 @@ void dfree(pmmm_plan* pl, P*& p) {
 }
 
 void free_particles(pmmm_plan* pl) {
-  dfree(pl, pl->sw.keys0);
-  dfree(pl, pl->sw.keys1);
-  dfree(pl, pl->sw.vals0);
-  dfree(pl, pl->sw.vals1);
-  dfree(pl, pl->sw.hist);
-  dfree(pl, pl->sw.chunks);
-  pl->sw = SortWork{};
+  dfree(pl, pl->keys);
+  dfree(pl, pl->keys_sorted);
+  dfree(pl, pl->vals_sorted);
+  dfree(pl, pl->order);
   dfree(pl, pl->part);
   dfree(pl, pl->far);
   dfree(pl, pl->item_cell);
@@ -82,7 +79,9 @@ void free_mesh(pmmm_plan* pl) {
   dfree(pl, pl->cs);
   dfree(pl, pl->corr);
   dfree(pl, pl->item_start);
-  dfree(pl, pl->item_chunks);
+  dfree(pl, pl->cell_count);
+  dfree(pl, pl->cs_local);
+  dfree(pl, pl->scan_tot);
   dfree(pl, pl->pair_start);
   dfree(pl, pl->energy);
   dfree(pl, pl->offsets_d);
@@ -140,9 +139,11 @@ cudaError_t alloc_mesh(pmmm_plan* pl, int B) {
   if (e == cudaSuccess) { e = dalloc(pl, &v, sizeof(int) * (size_t)(Kb + 1)); pl->cs = (int*)v; }
   if (e == cudaSuccess) { e = dalloc(pl, &v, sizeof(double) * 16 * (size_t)B); pl->corr = (double*)v; }
   if (e == cudaSuccess) { e = dalloc(pl, &v, sizeof(uint32_t) * (size_t)(Kb + 1)); pl->item_start = (uint32_t*)v; }
+  if (e == cudaSuccess) { e = dalloc(pl, &v, sizeof(uint32_t) * (size_t)Kb); pl->cell_count = (uint32_t*)v; }
+  if (e == cudaSuccess) { e = dalloc(pl, &v, sizeof(uint32_t) * (size_t)(Kb + 1)); pl->cs_local = (uint32_t*)v; }
   if (e == cudaSuccess) {
-    e = dalloc(pl, &v, sizeof(uint32_t) * (size_t)pp_lists_chunk_entries(Kb));
-    pl->item_chunks = (uint32_t*)v;
+    e = dalloc(pl, &v, sizeof(uint32_t) * (size_t)cell_list_totals(Kb));
+    pl->scan_tot = (uint32_t*)v;
   }
   if (e == cudaSuccess && !pl->fp64) {
     e = dalloc(pl, &v, sizeof(uint32_t) * (size_t)(Kb + 1));
@@ -152,6 +153,7 @@ cudaError_t alloc_mesh(pmmm_plan* pl, int B) {
   if (e == cudaSuccess) { e = dalloc(pl, &v, sizeof(int64_t) * (size_t)(B + 1)); pl->offsets_d = (int64_t*)v; }
   if (e == cudaSuccess) e = cudaMallocHost((void**)&pl->offsets_pinned, sizeof(int64_t) * (size_t)(B + 1));
   if (e == cudaSuccess) e = cudaMemsetAsync(pl->corr, 0, sizeof(double) * 16 * (size_t)B, pl->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(pl->cell_count, 0, sizeof(uint32_t) * (size_t)Kb, pl->stream);
   if (e == cudaSuccess) pl->bcap = B;
   return e;
 }
@@ -229,12 +231,10 @@ int ensure_particles(pmmm_plan* pl, int64_t n) {
     return map_cuda(e);                                 \
   }                                                     \
   field = (type*)v;
-  ALLOC(pl->sw.keys0, uint32_t, cap);
-  ALLOC(pl->sw.keys1, uint32_t, cap);
-  ALLOC(pl->sw.vals0, uint32_t, cap);
-  ALLOC(pl->sw.vals1, uint32_t, cap);
-  ALLOC(pl->sw.hist, uint32_t, sort_hist_entries(cap));
-  ALLOC(pl->sw.chunks, uint32_t, sort_chunk_entries(cap));
+  ALLOC(pl->keys, uint32_t, cap);
+  ALLOC(pl->keys_sorted, uint32_t, cap);
+  ALLOC(pl->vals_sorted, uint32_t, cap);
+  ALLOC(pl->order, uint32_t, cap + 4);
 #undef ALLOC
   e = dalloc(pl, &pl->part, 4 * pl->tsize * (size_t)cap);
   if (e == cudaSuccess) e = dalloc(pl, &pl->far, 4 * pl->tsize * (size_t)cap);
@@ -257,7 +257,6 @@ int ensure_particles(pmmm_plan* pl, int64_t n) {
     free_particles(pl);
     return map_cuda(e);
   }
-  pl->sw.cap = cap;
   pl->cap = cap;
   pl->max_items = mi;
   return PMMM_OK;
@@ -483,20 +482,21 @@ int run(pmmm_plan* pl, int B, int64_t n, const void* pos, const void* q, void* p
   } while (0)
   mark(pl, ST_SORT);
   {
-    int key_bits = 0;
-    while (((int64_t)1 << key_bits) < K) ++key_bits;
-    // the unsorted records go to `far`, which L2P overwrites later
-    if (B == 1)
-      CK(launch_bin(pos, q, fp64, n, pl->g, pl->sw.keys0, pl->far, pl->err, s, &nl));
-    else
-      CK(launch_bin_batched(pos, q, fp64, n, pl->offsets_d, B, pl->g, Ks, pl->sw.keys0, pl->far, pl->err, s, &nl));
-    CK(launch_radix_sort(pl->sw, n, key_bits, &pl->keys_sorted, &pl->vals_sorted, s, &nl));
-    CK(launch_cell_bounds(pl->keys_sorted, n, K, pl->cs, s, &nl));
-    CK(launch_pp_lists(pl->cs, K, pl->item_start, fp64 ? nullptr : pl->pair_start, pl->item_chunks, pl->counter, s,
-                       &nl));
-    CK(launch_gather_lists(pl->far, fp64, pl->vals_sorted, pl->keys_sorted, pl->cs, pl->item_start, pl->pair_start, n,
-                           K, pl->part, fp64 ? nullptr : pl->src2, pl->item_cell, pl->epart, pp_items_max(K, n),
-                           per_target, s, &nl));
+    CellLists cl;
+    cl.cs = pl->cs;
+    cl.cs_local = pl->cs_local;
+    cl.item_start = pl->item_start;
+    cl.pair_start = fp64 ? nullptr : pl->pair_start;
+    cl.tot = pl->scan_tot;
+    cl.ticket = pl->counter + 1;
+    cl.counter = pl->counter;
+    // the unsorted records go to `far`, which L2P overwrites later; the arrival numbers
+    // to vals_sorted, which the last step of the sort overwrites
+    CK(launch_bin_count(pos, q, fp64, n, B == 1 ? nullptr : pl->offsets_d, B, pl->g, Ks, pl->keys, pl->vals_sorted,
+                        pl->cell_count, pl->far, pl->err, s, &nl));
+    CK(launch_cell_sort(pl->keys, pl->vals_sorted, pl->cell_count, pl->far, fp64, n, K, cl, pl->order,
+                        pl->vals_sorted, pl->keys_sorted, pl->part, fp64 ? nullptr : pl->src2, pl->item_cell,
+                        pl->epart, pp_items_max(K, n), per_target, s, &nl));
   }
   // Split evaluation: the far field (P2M .. L2P) goes to the plan's second stream
   // and runs beside the near field, which then leaves its sums in nearv; a
@@ -614,6 +614,8 @@ int run(pmmm_plan* pl, int B, int64_t n, const void* pos, const void* q, void* p
 #undef CK
 done:
   if (split) set_streams(pl, s);
+  // a sequence that broke off may have left counts behind
+  if (e != cudaSuccess && !pl->capturing) cudaMemsetAsync(pl->cell_count, 0, sizeof(uint32_t) * (size_t)K, s);
   pl->split_last = split && e == cudaSuccess;
   pl->launches = nl;
   pl->n_last = n;
@@ -916,7 +918,8 @@ int pmmm_plan_create(const pmmm_config* cfg, void* stream, pmmm_plan** out) {
   // the reduction tickets at the end of partial start at zero
   if (e == cudaSuccess) e = cudaMemsetAsync(pl->partial, 0, sizeof(double) * 256 * 16, pl->stream);
   if (e == cudaSuccess) { e = dalloc(pl, &v, sizeof(int)); pl->err = (int*)v; }
-  if (e == cudaSuccess) { e = dalloc(pl, &v, sizeof(unsigned int)); pl->counter = (unsigned int*)v; }
+  if (e == cudaSuccess) { e = dalloc(pl, &v, 2 * sizeof(unsigned int)); pl->counter = (unsigned int*)v; }
+  if (e == cudaSuccess) e = cudaMemsetAsync(pl->counter, 0, 2 * sizeof(unsigned int), pl->stream);
   if (e == cudaSuccess) {
     int dev = 0;
     e = cudaGetDevice(&dev);

@@ -22,7 +22,7 @@ namespace {
 constexpr int PP_WARPS = 4;
 constexpr int PP_BATCH = 1;  // work items taken per atomic by the FP32 near-field warps (one: the shortest tail)
 constexpr int PP_BLOCKS_PER_SM = 6;  // resident blocks per SM (up to 80 registers per thread)
-constexpr int CHUNK = 32;
+constexpr int CHUNK = PP_CHUNK;
 
 template <typename T> struct V4;
 template <> struct V4<float> { using type = float4; };
@@ -42,178 +42,11 @@ template <typename T> __device__ __forceinline__ T rsq(T x);
 template <> __device__ __forceinline__ float rsq<float>(float x) { return rsqrt_ftz(x); }
 template <> __device__ __forceinline__ double rsq<double>(double x) { return rsqrt(x); }
 
-// item counts per cell: ceil(count / CHUNK)
-__global__ void item_count_kernel(const int* __restrict__ cs, int64_t K, uint32_t* __restrict__ item_start,
-                                  uint32_t* __restrict__ pair_start, unsigned int* __restrict__ counter) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c == 0) *counter = 0u;
-  if (c > K) return;
-  const int cnt = (c < K) ? cs[c + 1] - cs[c] : 0;
-  item_start[c] = (uint32_t)((cnt + CHUNK - 1) / CHUNK);
-  if (pair_start) pair_start[c] = (uint32_t)((cnt + 1) / 2);
-}
-
 // Pair-interleaved source records for the FP32 near field: the particles of
 // cell c occupy pairs pair_start[c] ... (a cell with an odd count ends with a
 // dummy of zero charge far outside the box).  Pair j is two 16-byte words
 // {x_a, x_b, y_a, y_b}, {z_a, z_b, q_a, q_b}, so that one 128-bit load yields
 // the packed operands of two sources.
-
-// Work lists: item and source-pair counts per cell from the cell offsets and
-// their exclusive prefix sums, in two launches of LIST_BLK cells per block
-// (lane = cell, loads and stores coalesced): list_local_kernel scans each block's
-// cells (warp scans, then a scan of the 32 warp totals) and writes the block
-// totals; list_fix_kernel adds to every cell the totals of the blocks before its
-// own (a warp sums at most LIST_MAX_BLOCKS of them).
-constexpr int LIST_BLK = 1024;
-constexpr int64_t LIST_MAX_BLOCKS = 1024;
-
-__device__ __forceinline__ void cell_counts(const int* __restrict__ cs, int64_t c, int64_t K, uint32_t& ni,
-                                            uint32_t& np) {
-  ni = np = 0u;
-  if (c < K) {
-    const int cnt = __ldg(cs + c + 1) - __ldg(cs + c);
-    ni = (uint32_t)((cnt + CHUNK - 1) / CHUNK);
-    np = (uint32_t)((cnt + 1) / 2);
-  }
-}
-
-__global__ void __launch_bounds__(LIST_BLK) list_local_kernel(const int* __restrict__ cs, int64_t K,
-                                                              uint32_t* __restrict__ item_start,
-                                                              uint32_t* __restrict__ pair_start,
-                                                              uint32_t* __restrict__ tot,
-                                                              unsigned int* __restrict__ counter) {
-  __shared__ uint32_t wi[32], wp[32];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t c = (int64_t)blockIdx.x * LIST_BLK + tid;
-  uint32_t a, q;
-  cell_counts(cs, c, K, a, q);
-  uint32_t ii = a, ip = q;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t x = __shfl_up_sync(0xffffffffu, ii, o), y = __shfl_up_sync(0xffffffffu, ip, o);
-    if (lane >= o) {
-      ii += x;
-      ip += y;
-    }
-  }
-  if (lane == 31) {
-    wi[warp] = ii;
-    wp[warp] = ip;
-  }
-  __syncthreads();
-  // exclusive offsets of the warps (every warp scans the 32 totals)
-  uint32_t ti = wi[lane], tp = wp[lane];
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t x = __shfl_up_sync(0xffffffffu, ti, o), y = __shfl_up_sync(0xffffffffu, tp, o);
-    if (lane >= o) {
-      ti += x;
-      tp += y;
-    }
-  }
-  const uint32_t oi = __shfl_sync(0xffffffffu, ti - wi[lane], warp);
-  const uint32_t op = __shfl_sync(0xffffffffu, tp - wp[lane], warp);
-  if (c <= K) {
-    item_start[c] = oi + ii - a;
-    if (pair_start) pair_start[c] = op + ip - q;
-  }
-  if (tid == LIST_BLK - 1) {
-    tot[2 * blockIdx.x] = __shfl_sync(0xffffffffu, ti, 31);
-    tot[2 * blockIdx.x + 1] = __shfl_sync(0xffffffffu, tp, 31);
-  }
-  if (c == 0) *counter = 0u;
-}
-
-__global__ void __launch_bounds__(LIST_BLK) list_fix_kernel(int64_t K, uint32_t* __restrict__ item_start,
-                                                            uint32_t* __restrict__ pair_start,
-                                                            const uint32_t* __restrict__ tot) {
-  __shared__ uint32_t pre[2];
-  const int b = blockIdx.x;
-  if (b == 0) return;  // the first block's sums are complete
-  if (threadIdx.x < 32) {
-    uint32_t si = 0u, sp = 0u;
-    for (int j = threadIdx.x; j < b; j += 32) {
-      si += tot[2 * j];
-      sp += tot[2 * j + 1];
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      si += __shfl_xor_sync(0xffffffffu, si, o);
-      sp += __shfl_xor_sync(0xffffffffu, sp, o);
-    }
-    if (threadIdx.x == 0) {
-      pre[0] = si;
-      pre[1] = sp;
-    }
-  }
-  __syncthreads();
-  const int64_t c = (int64_t)b * LIST_BLK + threadIdx.x;
-  if (c <= K) {
-    item_start[c] += pre[0];
-    if (pair_start) pair_start[c] += pre[1];
-  }
-}
-
-// Sorted records part[s] = rec[vals[s]] (a pure permutation), and with them the
-// near-field work lists: the cell of every work item (the first particle of each
-// chunk of CHUNK writes it), the pair-interleaved FP32 sources (PACK, layout
-// above) and zeroed energy partials of the unused item slots (of all
-// slots when the near-field kernel accumulates into them).
-template <typename V, bool PACK>
-__global__ void gather_lists_kernel(const V* __restrict__ rec, const uint32_t* __restrict__ vals,
-                                    const uint32_t* __restrict__ keys, const int* __restrict__ cs,
-                                    const uint32_t* __restrict__ item_start, const uint32_t* __restrict__ pair_start,
-                                    int64_t n, int64_t K, V* __restrict__ part, float* __restrict__ src2,
-                                    uint32_t* __restrict__ item_cell, double* __restrict__ epart, int64_t max_items,
-                                    int zero_all) {
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  for (int64_t i = (zero_all ? 0 : (int64_t)item_start[K]) + s; i < max_items; i += (int64_t)gridDim.x * blockDim.x)
-    epart[4 * i] = epart[4 * i + 1] = epart[4 * i + 2] = epart[4 * i + 3] = 0.0;
-  if (s - (int64_t)(threadIdx.x & 31) >= n) return;  // the whole warp lies past the particles
-  const bool live = s < n;  // lanes past the particles stay for the shuffles below
-  V r;
-  r.x = r.y = r.z = r.w = 0;
-  uint32_t cell = 0;
-  int j = 0;
-  if (live) {
-    r = rec[vals[s]];
-    part[s] = r;
-    cell = keys[s];
-    j = (int)(s - cs[cell]);
-    if (j % CHUNK == 0) item_cell[item_start[cell] + j / CHUNK] = cell;
-  }
-  if constexpr (PACK) {
-    // pair record of (a, b) = sorted particles (s, s + 1), j even: a writes
-    // {x_a, x_b, y_a, y_b}, b writes {z_a, z_b, q_a, q_b}, each one 16-byte store; the
-    // partner's values come from the neighbouring lane (a global load at the warp's edge)
-    const int slot = j & 1;
-    const int lane = threadIdx.x & 31;
-    const int src_lane = (slot == 0 ? lane + 1 : lane - 1) & 31;
-    float px = __shfl_sync(0xffffffffu, (float)r.x, src_lane), py = __shfl_sync(0xffffffffu, (float)r.y, src_lane);
-    float pz = __shfl_sync(0xffffffffu, (float)r.z, src_lane), pw = __shfl_sync(0xffffffffu, (float)r.w, src_lane);
-    if (!live) return;
-    const int64_t pj = (int64_t)pair_start[cell] + j / 2;
-    const bool alone = slot == 0 && s + 1 == (int64_t)cs[cell + 1];  // odd count: dummy partner
-    const bool edge = slot == 0 ? lane == 31 : lane == 0;  // partner in the neighbouring warp
-    if (alone) {
-      px = py = pz = 1.0e4f;
-      pw = 0.0f;
-    } else if (edge) {
-      const V pr = rec[vals[slot == 0 ? s + 1 : s - 1]];
-      px = (float)pr.x;
-      py = (float)pr.y;
-      pz = (float)pr.z;
-      pw = (float)pr.w;
-    }
-    float4* o = reinterpret_cast<float4*>(src2 + 8 * pj);
-    if (slot == 0)
-      o[0] = make_float4((float)r.x, px, (float)r.y, py);
-    else
-      o[1] = make_float4(pz, (float)r.z, pw, (float)r.w);
-    if (alone) o[1] = make_float4((float)r.z, pz, (float)r.w, pw);
-  }
-}
 
 // Accumulates the interactions of target (tx, ty, tz) with sources P[b + e],
 // e = ph, ph + SP, ... < cnt.  SELF: the source set may contain the target
@@ -274,7 +107,7 @@ template <> struct PPConst<double> {
 __device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 
 // Persistent warps: each takes work items from a global counter (reset to zero
-// by the work-list kernels) until all are done.  Every item's results depend
+// by the cell sort) until all are done.  Every item's results depend
 // only on the item, so the assignment order does not change any output bit.
 // NB_SLOTS: neighbour-table slots per lane, (2c+1)^3 <= 32 * NB_SLOTS (1 for c = 1, 4 for c = 2)
 template <typename T, int NB_SLOTS>
@@ -996,52 +829,6 @@ __global__ void __launch_bounds__(PPS_THREADS, 4) pp_target_kernel(
 int64_t pp_items_max(int64_t K, int64_t n) { return K + (n + CHUNK - 1) / CHUNK + 1; }
 
 int64_t pp_pairs_max(int64_t K, int64_t n) { return (n + K) / 2 + 1; }
-
-int64_t pp_lists_chunk_entries(int64_t K) {
-  const int64_t a = scan_chunk_count(K + 1), b = 2 * ((K + 1 + LIST_BLK - 1) / LIST_BLK);
-  return a > b ? a : b;
-}
-
-cudaError_t launch_pp_lists(const int* cell_start, int64_t K, uint32_t* item_start, uint32_t* pair_start,
-                            uint32_t* chunks, unsigned int* counter, cudaStream_t s, int* nl) {
-  const int64_t nb = (K + 1 + LIST_BLK - 1) / LIST_BLK;
-  if (nb <= LIST_MAX_BLOCKS) {
-    list_local_kernel<<<(unsigned)nb, LIST_BLK, 0, s>>>(cell_start, K, item_start, pair_start, chunks, counter);
-    ++*nl;
-    if (nb > 1) {
-      list_fix_kernel<<<(unsigned)nb, LIST_BLK, 0, s>>>(K, item_start, pair_start, chunks);
-      ++*nl;
-    }
-    return cudaGetLastError();
-  }
-  item_count_kernel<<<(unsigned)((K + 1 + 255) / 256), 256, 0, s>>>(cell_start, K, item_start, pair_start, counter);
-  ++*nl;
-  cudaError_t e = launch_exclusive_scan(item_start, K + 1, chunks, s, nl);
-  if (e == cudaSuccess && pair_start) e = launch_exclusive_scan(pair_start, K + 1, chunks, s, nl);
-  return e;
-}
-
-cudaError_t launch_gather_lists(const void* rec, bool fp64, const uint32_t* vals, const uint32_t* keys,
-                                const int* cell_start, const uint32_t* item_start, const uint32_t* pair_start,
-                                int64_t n, int64_t K, void* part, void* src2, uint32_t* item_cell, double* epart,
-                                int64_t max_items, bool zero_all, cudaStream_t s, int* nl) {
-  const int64_t work = n > max_items ? n : max_items;
-  const unsigned blocks = (unsigned)((work + 255) / 256 > 0 ? (work + 255) / 256 : 1);
-  if (fp64)
-    gather_lists_kernel<double4, false><<<blocks, 256, 0, s>>>((const double4*)rec, vals, keys, cell_start, item_start,
-                                                                 pair_start, n, K, (double4*)part, nullptr, item_cell,
-                                                                 epart, max_items, zero_all ? 1 : 0);
-  else if (src2)
-    gather_lists_kernel<float4, true><<<blocks, 256, 0, s>>>((const float4*)rec, vals, keys, cell_start, item_start,
-                                                               pair_start, n, K, (float4*)part, (float*)src2,
-                                                               item_cell, epart, max_items, zero_all ? 1 : 0);
-  else
-    gather_lists_kernel<float4, false><<<blocks, 256, 0, s>>>((const float4*)rec, vals, keys, cell_start, item_start,
-                                                                pair_start, n, K, (float4*)part, nullptr, item_cell,
-                                                                epart, max_items, zero_all ? 1 : 0);
-  ++*nl;
-  return cudaGetLastError();
-}
 
 bool pp_per_target_applies(bool fp64, int c) { return !fp64 && c <= 2; }
 bool pp_tma_applies(bool fp64, int c, bool per_target) { return !fp64 && c <= 2 && !per_target; }

@@ -1,5 +1,6 @@
-// Binning and stable counting sort of the particles by cell (Sec. 2.1: "for
-// each cell, the set of particles inside is known ... in an O(N) procedure").
+// Binning and stable radix sort of the particles by cell, for the allocation-free
+// entry point (static_sort.cu): its scratch is a fixed array, without the counter per
+// cell that the sort of the evaluations (cellsort.cu) uses.
 //
 // Cell index, in FP64 with every operation rounded (no contraction):
 //   t = x - lo;  if t is outside [0, len):
@@ -216,29 +217,12 @@ __global__ void cell_bounds_kernel(const uint32_t* __restrict__ keys, int64_t n,
   for (int64_t c = kprev + 1; c <= k; ++c) cs[c] = (int)s;
 }
 
-__global__ void scan_add_kernel(uint32_t* __restrict__ data, int64_t n, const uint32_t* __restrict__ chunks) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) data[i] += chunks[i / SCAN_CH];
-}
-
 inline int grid1(int64_t n, int b) { return (int)((n + b - 1) / b); }
 }  // namespace
 
-int64_t scan_chunk_count(int64_t n) { return (n + SCAN_CH - 1) / SCAN_CH + 1; }
-
-cudaError_t launch_exclusive_scan(uint32_t* data, int64_t n, uint32_t* chunks, cudaStream_t s, int* nl) {
-  if (n <= 0) return cudaSuccess;
-  const int nchunks = (int)((n + SCAN_CH - 1) / SCAN_CH);
-  scan_chunks_kernel<<<nchunks, SCAN_THREADS, 0, s>>>(data, n, chunks);
-  scan_top_kernel<<<1, SCAN_THREADS, 0, s>>>(chunks, nchunks);
-  scan_add_kernel<<<grid1(n, 256), 256, 0, s>>>(data, n, chunks);
-  *nl += 3;
-  return cudaGetLastError();
-}
-
+namespace {
 int sort_tiles(int64_t n) { return (int)((n + RS_TILE - 1) / RS_TILE); }
-size_t sort_hist_entries(int64_t n) { return (size_t)256 * (size_t)(sort_tiles(n) > 0 ? sort_tiles(n) : 1); }
-size_t sort_chunk_entries(int64_t n) { return (sort_hist_entries(n) + SCAN_CH - 1) / SCAN_CH + 1; }
+}  // namespace
 
 cudaError_t launch_bin(const void* pos, const void* q, bool fp64, int64_t n, const Geo& g, uint32_t* keys, void* rec,
                        int* err, cudaStream_t s, int* nl) {
