@@ -129,7 +129,9 @@ cudaError_t launch_cell_bounds(const uint32_t* keys, int64_t n, int64_t K, int* 
                                int* nlaunch);
 
 // ---------------------------------------------------------------- p2m_l2p.cu
-// sparse (FP32, p <= 8): one thread per cell, crowded cells taken by the whole warp
+// sparse (FP32, p <= 8): one thread per cell, crowded cells taken by the whole warp;
+// for systems of fewer than P2M_SPARSE particles per cell
+constexpr int64_t P2M_SPARSE = 8;
 cudaError_t launch_p2m(int p, bool fp64, const void* part, const int* cell_start, int64_t K, void* M,
                        double* cellq, double* celld, bool sparse, cudaStream_t s, int* nlaunch);
 struct CorrParams {

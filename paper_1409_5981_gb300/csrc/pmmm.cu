@@ -468,7 +468,11 @@ int run(pmmm_plan* pl, int B, int64_t n, const void* pos, const void* q, void* p
   const bool fp64 = pl->fp64;
   const int64_t Ks = pl->d.K, K = Ks * B;  // cells per system, cells of all systems
   // near field: one thread per target when asked, or (automatic) when the cells
-  // hold fewer than PMMM_NEAR_AUTO_OCCUPANCY particles on average
+  // hold fewer than PMMM_NEAR_AUTO_OCCUPANCY particles on average: the two kernels
+  // take the same time on uniform systems of 16 to 17 (c = 1) and 16 (c = 2) particles
+  // per cell (2^15 cells, c = 1: 12 per cell 133 us per target, 164 us items; 16: 209
+  // and 219 us; 24: 416 and 358 us).  Crowded cells of an uneven system cost the
+  // per-target kernel 1.2 times the items' time, no more
   const bool sparse = n < (int64_t)PMMM_NEAR_AUTO_OCCUPANCY * K;
   const int near = pl->tuned_near ? pl->tuned_near : pl->cfg.near_field;
   const bool per_target = pp_per_target_applies(fp64, pl->g.c) &&
@@ -523,7 +527,7 @@ int run(pmmm_plan* pl, int B, int64_t n, const void* pos, const void* q, void* p
     set_streams(pl, fs);
   }
   mark(pl, ST_P2M);
-  CK(launch_p2m(pl->p, fp64, pl->part, pl->cs, K, pl->M, pl->cellsum, pl->cellsum + K, sparse, fs, &nl));
+  CK(launch_p2m(pl->p, fp64, pl->part, pl->cs, K, pl->M, pl->cellsum, pl->cellsum + K, n < P2M_SPARSE * K, fs, &nl));
   mark(pl, ST_FFT_FWD);
   CK(pl->hier ? hier_stage(pl, &nl) : mesh_stage(pl, B, &nl));
   mark(pl, ST_L2P);

@@ -704,14 +704,82 @@ __global__ void __launch_bounds__(256) pp_combine_kernel(const float4* __restric
 
 // FP32 near field (c = 1 or 2) with one thread per target: for sparsely filled cells,
 // where the per-item set-up of the cell-item kernels costs more than the
-// interactions.  Thread i takes sorted target i; it walks the 9 neighbour rows
-// (dy, dz) and in each row the pairs of the cells x-1, x, x+1 of the pair layout
-// (sources of neighbouring targets coincide, so loads are served by L1).  Energy
+// interactions.  Thread i takes sorted target i; it walks the (2c+1)^2 neighbour rows
+// (dy, dz) and in each row the source pairs of its 2c+1 cells x-c .. x+c as one list,
+// two pairs per step (sources of neighbouring targets coincide, so loads are served by
+// L1).  One loop per row instead of one per cell: the lanes of a warp wait for each
+// other 9 (25) times instead of 27 (125), and row totals of neighbouring targets, which
+// share most of their cells, are more alike than cell counts.  A warp whose 32 targets
+// lie in one cell (a crowded one) takes its sources through shared memory instead, 32
+// pairs of a neighbour cell at a time: the broadcast loads then come from there, at
+// twice the rate of L1, and need no per-lane addresses.  Same pairs in the same order
+// with the same rounding.  Bound by latency and divergence where cells are sparse, by
+// the pair step's operand reads (33 cycles per 64 pairs and SM quarter) where they are
+// full.  Against one loop per cell and L1 loads throughout: 20011 particles / 16^3 29 ->
+// 20 us; 10^6 / 64^3 195 -> 160 us; 5.6 million in 64 systems 1336 -> 1124 us; 2^20 in a
+// Plummer sphere / 64^3 (3.5e10 pairs, up to 6300 particles per cell) 27.9 -> 18.4 ms.  Energy
 // and net-force terms are reduced per work item: a segmented warp scan over
 // lanes of equal item, one store per item that lies inside the warp, and two
 // double atomics (commutative, so deterministic) on a zeroed slot for an item
 // split between two warps.
 constexpr int PPS_THREADS = 256;
+
+// Sums of one target over npair pairs whose words lie in sa and sb (shared memory).
+template <bool SELF>
+__device__ __forceinline__ void pp_staged(const float4* __restrict__ sa, const float4* __restrict__ sb, int npair,
+                                          float2 tx, float2 ty, float2 tz, float2& pot, float2& gx, float2& gy,
+                                          float2& gz) {
+  int j = 0;
+  for (; j + 4 <= npair; j += 4) {
+    float4 A[4], B[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      A[u] = sa[j + u];
+      B[u] = sb[j + u];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) pp_pair_v<SELF>(A[u], B[u], tx, ty, tz, pot, gx, gy, gz);
+  }
+  for (; j < npair; ++j) pp_pair_v<SELF>(sa[j], sb[j], tx, ty, tz, pot, gx, gy, gz);
+}
+
+// The near sums of 32 targets of one cell (lane = target): pot, g of pp_target_kernel.
+template <int CUT>
+__device__ __forceinline__ void pp_crowd_warp(const float4 xi, int sbase, int ix, int iy, int iz,
+                                              const float4* __restrict__ S2, const uint32_t* __restrict__ pair_start,
+                                              const PPParams& pp, float4* sa, float4* sb, float2& pot, float2& gx,
+                                              float2& gy, float2& gz) {
+  const int lane = threadIdx.x & 31;
+  for (int dz = -CUT; dz <= CUT; ++dz)
+    for (int dy = -CUT; dy <= CUT; ++dy)
+      for (int dx = -CUT; dx <= CUT; ++dx) {
+        int jx = ix + dx, jy = iy + dy, jz = iz + dz;
+        bool ok = true;
+        if (jx < 0 || jx >= pp.n[0]) { ok = ok && pp.periodic; jx += (jx < 0) ? pp.n[0] : -pp.n[0]; }
+        if (jy < 0 || jy >= pp.n[1]) { ok = ok && pp.periodic; jy += (jy < 0) ? pp.n[1] : -pp.n[1]; }
+        if (jz < 0 || jz >= pp.n[2]) { ok = ok && pp.periodic; jz += (jz < 0) ? pp.n[2] : -pp.n[2]; }
+        if (!ok) continue;
+        const uint32_t* row = pair_start + sbase + jx + pp.n[0] * (jy + pp.n[1] * jz);
+        const int pb = (int)__ldg(row), pe = (int)__ldg(row + 1);
+        const float ux = xi.x - (float)dx * pp.cs32[0], uy = xi.y - (float)dy * pp.cs32[1],
+                    uz = xi.z - (float)dz * pp.cs32[2];
+        const float2 tx = make_float2(ux, ux), ty = make_float2(uy, uy), tz = make_float2(uz, uz);
+        const bool own = dx == 0 && dy == 0 && dz == 0;
+        for (int p = pb; p < pe; p += 32) {
+          const int m = min(32, pe - p);
+          __syncwarp();
+          if (lane < m) {
+            sa[lane] = __ldg(S2 + 2 * (int64_t)(p + lane));
+            sb[lane] = __ldg(S2 + 2 * (int64_t)(p + lane) + 1);
+          }
+          __syncwarp();
+          if (own)
+            pp_staged<true>(sa, sb, m, tx, ty, tz, pot, gx, gy, gz);
+          else
+            pp_staged<false>(sa, sb, m, tx, ty, tz, pot, gx, gy, gz);
+        }
+      }
+}
 
 template <int CUT>
 __global__ void __launch_bounds__(PPS_THREADS, 4) pp_target_kernel(
@@ -719,15 +787,20 @@ __global__ void __launch_bounds__(PPS_THREADS, 4) pp_target_kernel(
     const uint32_t* __restrict__ keys, const uint32_t* __restrict__ vals, const int* __restrict__ cs,
     const uint32_t* __restrict__ item_start, int64_t n, const float4* __restrict__ far, PPParams pp,
     float* __restrict__ phi, float* __restrict__ force, double* __restrict__ epart) {
+  constexpr int W = 2 * CUT + 1;
   const int64_t i = (int64_t)blockIdx.x * PPS_THREADS + threadIdx.x;
   const int lane = threadIdx.x & 31;
   const int64_t wbase = i - lane;
   float e_t = 0.f, f_t0 = 0.f, f_t1 = 0.f, f_t2 = 0.f;
   uint32_t item = 0xffffffffu;
   int64_t tb = 0, te = 0;
+  __shared__ float4 stage[PPS_THREADS / 32][2][32];
+  const int mycell = i < n ? (int)keys[i] : -1;
+  const int cell0 = __shfl_sync(0xffffffffu, mycell, 0);  // every lane takes part
+  const bool crowd = __all_sync(0xffffffffu, mycell >= 0 && mycell == cell0);
   if (i < n) {
     const float4 xi = P[i];
-    const int cell = (int)keys[i];
+    const int cell = mycell;
     const int c0 = cs[cell], c1 = cs[cell + 1];
     const int chunk = (int)((i - c0) / CHUNK);
     item = item_start[cell] + (uint32_t)chunk;
@@ -737,45 +810,84 @@ __global__ void __launch_bounds__(PPS_THREADS, 4) pp_target_kernel(
     const int sbase = cell - cell % pp.ksys, lc = cell - sbase;
     const int ix = lc % nx, iy = (lc / nx) % ny, iz = lc / (nx * ny);
     const float csx = pp.cs32[0], csy = pp.cs32[1], csz = pp.cs32[2];
-    f2 pot = pk2(0.f, 0.f), gx = pot, gy = pot, gz = pot;
-    for (int dz = -CUT; dz <= CUT; ++dz) {
-      int jz = iz + dz;
-      if (jz < 0 || jz >= nz) {
-        if (!pp.periodic) continue;
-        jz += (jz < 0) ? nz : -nz;
-      }
-      const float tzs = xi.z - (float)dz * csz;
-      const f2 tz = pk2(tzs, tzs);
-      for (int dy = -CUT; dy <= CUT; ++dy) {
-        int jy = iy + dy;
-        if (jy < 0 || jy >= ny) {
-          if (!pp.periodic) continue;
-          jy += (jy < 0) ? ny : -ny;
-        }
-        const float tys = xi.y - (float)dy * csy;
-        const f2 ty = pk2(tys, tys);
-        const int row = sbase + nx * (jy + ny * jz);
+    float pa = 0.f, pbv = 0.f, xa = 0.f, xb = 0.f, ya = 0.f, yb = 0.f, za = 0.f, zb = 0.f;
+    if (crowd) {
+      float2 pot = make_float2(0.f, 0.f), gx = pot, gy = pot, gz = pot;
+      float4(*st)[32] = stage[threadIdx.x >> 5];
+      pp_crowd_warp<CUT>(xi, sbase, ix, iy, iz, reinterpret_cast<const float4*>(S2), pair_start, pp, st[0], st[1], pot,
+                         gx, gy, gz);
+      pa = pot.x; pbv = pot.y; xa = gx.x; xb = gx.y; ya = gy.x; yb = gy.y; za = gz.x; zb = gz.y;
+    } else {
+      f2 pot = pk2(0.f, 0.f), gx = pot, gy = pot, gz = pot;
+      // the row's cells: x index (wrapped; -1 outside an open box) and the target's x there
+      int jx[W];
+      float txs[W];
 #pragma unroll
-        for (int d = 0; d < 2 * CUT + 1; ++d) {
-          int jx = ix + d - CUT;
-          if (jx < 0 || jx >= nx) {
+      for (int d = 0; d < W; ++d) {
+        jx[d] = ix + d - CUT;
+        if (jx[d] < 0 || jx[d] >= nx) jx[d] = pp.periodic ? jx[d] + (jx[d] < 0 ? nx : -nx) : -1;
+        txs[d] = xi.x - (float)(d - CUT) * csx;
+      }
+      for (int dz = -CUT; dz <= CUT; ++dz) {
+        int jz = iz + dz;
+        if (jz < 0 || jz >= nz) {
+          if (!pp.periodic) continue;
+          jz += (jz < 0) ? nz : -nz;
+        }
+        const float tzs = xi.z - (float)dz * csz;
+        const f2 tz = pk2(tzs, tzs);
+        for (int dy = -CUT; dy <= CUT; ++dy) {
+          int jy = iy + dy;
+          if (jy < 0 || jy >= ny) {
             if (!pp.periodic) continue;
-            jx += (jx < 0) ? nx : -nx;
+            jy += (jy < 0) ? ny : -ny;
           }
-          const int pb = (int)__ldg(pair_start + row + jx), pe = (int)__ldg(pair_start + row + jx + 1);
-          const float txs = xi.x - (float)(d - CUT) * csx;
-          const f2 tx = pk2(txs, txs);
-#pragma unroll 1
-          for (int pr = pb; pr < pe; ++pr)
-            pp_pair2_mixed<true>(S2[2 * pr], S2[2 * pr + 1], tx, ty, tz, pot, gx, gy, gz);
+          const float tys = xi.y - (float)dy * csy;
+          const f2 ty = pk2(tys, tys);
+          const uint32_t* row = pair_start + sbase + nx * (jy + ny * jz);
+          // list position e of cell d's pairs: first[d] <= e < first[d + 1], pair e + off[d]
+          int first[W], off[W], tot = 0;
+#pragma unroll
+          for (int d = 0; d < W; ++d) {
+            const int b = jx[d] >= 0 ? (int)__ldg(row + jx[d]) : 0;
+            const int m = jx[d] >= 0 ? (int)__ldg(row + jx[d] + 1) - b : 0;
+            first[d] = tot;
+            off[d] = b - tot;
+            tot += m;
+          }
+          auto at = [&](int e, const ulonglong2*& src, f2& tx) {
+            int o = off[0];
+            float t = txs[0];
+#pragma unroll
+            for (int d = 1; d < W; ++d)
+              if (e >= first[d]) {
+                o = off[d];
+                t = txs[d];
+              }
+            src = S2 + 2 * (int64_t)(e + o);
+            tx = pk2(t, t);
+          };
+          const ulonglong2 *s0, *s1;
+          f2 tx0, tx1;
+          int e = 0;
+          for (; e + 2 <= tot; e += 2) {
+            at(e, s0, tx0);
+            at(e + 1, s1, tx1);
+            const ulonglong2 A0 = s0[0], B0 = s0[1], A1 = s1[0], B1 = s1[1];
+            pp_pair2_mixed<true>(A0, B0, tx0, ty, tz, pot, gx, gy, gz);
+            pp_pair2_mixed<true>(A1, B1, tx1, ty, tz, pot, gx, gy, gz);
+          }
+          if (e < tot) {
+            at(e, s0, tx0);
+            pp_pair2_mixed<true>(s0[0], s0[1], tx0, ty, tz, pot, gx, gy, gz);
+          }
         }
       }
+      up2(pot, pa, pbv);
+      up2(gx, xa, xb);
+      up2(gy, ya, yb);
+      up2(gz, za, zb);
     }
-    float pa, pbv, xa, xb, ya, yb, za, zb;
-    up2(pot, pa, pbv);
-    up2(gx, xa, xb);
-    up2(gy, ya, yb);
-    up2(gz, za, zb);
     const float ps = pa + pbv, gxs = -(xa + xb), gys = -(ya + yb), gzs = -(za + zb);
     const float4 fr = far[i];
     const float ih = pp.ih32, ih2 = pp.ih2_32, sg = pp.sign32;
