@@ -280,18 +280,29 @@ struct GemmArgs {
   int64_t ldd = 0;
   __nv_bfloat16* D16 = nullptr;
   int64_t ldd16 = 0;
+  __nv_bfloat16* D16T = nullptr;  // with D16: its transpose, [column][row]
+  int64_t ldd16t = 0;
   const float* Zin = nullptr;
   int64_t ldz = 0;
   int epi = GEMM_EPI_LINEAR;
   int* err = nullptr;
 };
-cudaError_t launch_gemm_tc(const GemmArgs& a, cudaStream_t s, int* nlaunch);
+cudaError_t launch_gemm_tc(const GemmArgs& a, int num_sms, cudaStream_t s, int* nlaunch);
+// The gradients of three layers: weights g[p].D32 (contiguous, M x N) = the product g[p]
+// over K = rows, biases bout[p] = column sums of dz[p] [rows][cols[p]], and *loss =
+// loss_scale times the sum of the nloss loss parts.  wpart: weight_grad_slices(rows) times the
+// weights' elements; bpart: as many times the bias columns.
+int weight_grad_slices(int64_t rows);
+cudaError_t launch_weight_grads(const GemmArgs g[3], const float* const dz[3], const int cols[3], float* const bout[3],
+                                int rows, float* wpart, double* bpart, const double* loss_part, int nloss,
+                                double loss_scale, double* loss, cudaStream_t s, int* nlaunch);
 cudaError_t launch_transpose_bf16(const void* in, int64_t ld_in, void* out, int64_t ld_out, int R, int C,
                                   cudaStream_t s, int* nlaunch);
-cudaError_t launch_colsum(const float* in, int64_t ld, int R, int C, float* out, cudaStream_t s, int* nlaunch);
-// dO = 2 (O - T) / (rows nout) on columns < nout; *loss = mean square (device, FP64); part: nparts doubles
-cudaError_t launch_mse_grad(const float* O, const float* T, int64_t rows, int ld, int nout, float* dO, void* dO16,
-                            double* part, int nparts, double* loss, cudaStream_t s, int* nlaunch);
+// dO = 2 (O - T) / (rows nout) on columns < nout of [rows][128], FP32, BF16 and BF16
+// transposed; part: mse_grad_parts(rows) partial sums of (O - T)^2
+int mse_grad_parts(int64_t rows);
+cudaError_t launch_mse_grad(const float* O, const float* T, int64_t rows, int nout, float* dO, void* dO16, void* dO16T,
+                            double* part, cudaStream_t s, int* nlaunch);
 cudaError_t launch_adam(float* p, const float* g, float* m, float* v, int64_t n, float lr, int64_t step,
                         cudaStream_t s, int* nlaunch);
 cudaError_t launch_to_bf16(const float* in, void* out, int64_t n, cudaStream_t s, int* nlaunch);

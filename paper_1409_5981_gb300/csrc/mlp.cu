@@ -45,22 +45,21 @@ __device__ __forceinline__ uint32_t chunk_off(int r, int g) {
   return (uint32_t)(r >> 3) * G_SBO + (uint32_t)g * G_LBO + (uint32_t)(r & 7) * 16;
 }
 
-template <int TN>
-__global__ void __launch_bounds__(G_THREADS) gemm_tc_kernel(GemmArgs a) {
+// One 128 x TN tile (rows m0 .., columns n0 ..) of D over the K range [kbeg, kend),
+// written to D32 (row stride a.ldd) and, converted, to D16 / D16T.
+template <int TN, int ST>
+__device__ __forceinline__ void gemm_tile(const GemmArgs& a, int64_t m0, int n0, int kbeg, int kend,
+                                          float* __restrict__ D32) {
   constexpr uint32_t B_BYTES = TN * G_KC * 2;
   constexpr uint32_t STAGE = G_A_BYTES + B_BYTES;
   extern __shared__ __align__(1024) unsigned char smem[];
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + 2 * STAGE);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + 2 * STAGE + 16);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + ST * STAGE);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + ST * STAGE + 8 * ST);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t m0 = (int64_t)blockIdx.x * 128;
-  const int n0 = blockIdx.y * TN;
-  const int nchunks = (a.K + G_KC - 1) / G_KC;
+  const int nchunks = (kend - kbeg + G_KC - 1) / G_KC;
   const uint32_t sbase = tc::smem_u32(smem);
-
   if (tid == 0) {
-    tc::bar_init(tc::smem_u32(&bars[0]), 1);
-    tc::bar_init(tc::smem_u32(&bars[1]), 1);
+    for (int i = 0; i < ST; ++i) tc::bar_init(tc::smem_u32(&bars[i]), 1);
     tc::fence_proxy_async();
   }
   if (warp == 0) tc::tmem_alloc(tmem_slot, TN);
@@ -69,35 +68,30 @@ __global__ void __launch_bounds__(G_THREADS) gemm_tc_kernel(GemmArgs a) {
   tc::fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  auto load = [&](int ch, int st) {
-    const int k0 = ch * G_KC;
+  auto load = [&](int ch) {
+    const int k0 = kbeg + ch * G_KC, st = ch % ST;
     const uint32_t sa = sbase + st * STAGE, sb = sa + G_A_BYTES;
     for (int pi = tid; pi < 128 * 8; pi += G_THREADS) {
       const int r = pi >> 3, g = pi & 7, k = k0 + 8 * g;
-      const bool ok = k < a.K;
+      const bool ok = k < kend;
       cp16(sa + chunk_off(r, g), ok ? (const void*)(a.A + (m0 + r) * a.lda + k) : (const void*)a.A, ok);
     }
     for (int pi = tid; pi < TN * 8; pi += G_THREADS) {
       const int r = pi >> 3, g = pi & 7, k = k0 + 8 * g;
-      const bool ok = k < a.K && n0 + r < a.N;
+      const bool ok = k < kend && n0 + r < a.N;
       cp16(sb + chunk_off(r, g), ok ? (const void*)(a.B + (int64_t)(n0 + r) * a.ldb + k) : (const void*)a.B, ok);
     }
-    cp_commit();
   };
 
   bool ok = true;
-  load(0, 0);
   const uint32_t idesc = tc::idesc_bf16_m128(TN);
+  for (int ch = 0; ch < ST - 1; ++ch) {
+    if (ch < nchunks) load(ch);
+    cp_commit();
+  }
   for (int ch = 0; ch < nchunks; ++ch) {
-    const int st = ch & 1;
-    if (ch + 1 < nchunks) {
-      // the other stage was read by the MMAs of chunk ch - 1
-      if (ch >= 1 && !tc::bar_wait(tc::smem_u32(&bars[st ^ 1]), (uint32_t)(((ch - 1) >> 1) & 1), G_WAIT_LIMIT)) ok = false;
-      load(ch + 1, st ^ 1);
-      cp_wait<1>();
-    } else {
-      cp_wait<0>();
-    }
+    const int st = ch % ST;
+    cp_wait<ST - 2>();  // this thread's copies of chunk ch
     tc::fence_proxy_async();
     __syncthreads();
     if (tid == 0) {
@@ -109,10 +103,18 @@ __global__ void __launch_bounds__(G_THREADS) gemm_tc_kernel(GemmArgs a) {
                      (ch | j) != 0);
       tc::commit(tc::smem_u32(&bars[st]));
     }
+    const int nx = ch + ST - 1;  // goes into the stage that the MMAs of chunk ch - 1 read
+    if (nx < nchunks) {
+      if (ch >= 1 &&
+          !tc::bar_wait(tc::smem_u32(&bars[(ch - 1) % ST]), (uint32_t)(((ch - 1) / ST) & 1), G_WAIT_LIMIT))
+        ok = false;
+      load(nx);
+    }
+    cp_commit();
   }
   const int last = nchunks - 1;
-  if (!__all_sync(0xffffffffu, tc::bar_wait(tc::smem_u32(&bars[last & 1]), (uint32_t)((last >> 1) & 1), G_WAIT_LIMIT)))
-    ok = false;
+  const bool done = tc::bar_wait(tc::smem_u32(&bars[last % ST]), (uint32_t)((last / ST) & 1), G_WAIT_LIMIT);
+  if (!__all_sync(0xffffffffu, done)) ok = false;
   tc::fence_after();
   if (__all_sync(0xffffffffu, ok)) {
     const int64_t row = m0 + 32 * warp + lane;
@@ -137,8 +139,8 @@ __global__ void __launch_bounds__(G_THREADS) gemm_tc_kernel(GemmArgs a) {
           v[4 * q + 3] *= gelu_prime(z.w);
         }
       }
-      if (a.D32) {
-        float4* dp = reinterpret_cast<float4*>(a.D32 + row * a.ldd + col);
+      if (D32) {
+        float4* dp = reinterpret_cast<float4*>(D32 + row * a.ldd + col);
 #pragma unroll
         for (int q = 0; q < 4; ++q) dp[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
       }
@@ -157,6 +159,14 @@ __global__ void __launch_bounds__(G_THREADS) gemm_tc_kernel(GemmArgs a) {
         uint4* hp = reinterpret_cast<uint4*>(a.D16 + row * a.ldd16 + col);
         hp[0] = make_uint4(h[0], h[1], h[2], h[3]);
         hp[1] = make_uint4(h[4], h[5], h[6], h[7]);
+        if (a.D16T) {  // the transpose: the warp's 32 rows are consecutive
+          unsigned short* tp = reinterpret_cast<unsigned short*>(a.D16T) + (int64_t)col * a.ldd16t + row;
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            tp[(int64_t)(2 * q) * a.ldd16t] = (unsigned short)(h[q] & 0xffffu);
+            tp[(int64_t)(2 * q + 1) * a.ldd16t] = (unsigned short)(h[q] >> 16);
+          }
+        }
       }
     }
   } else if (tid == 0 && a.err) {
@@ -165,6 +175,33 @@ __global__ void __launch_bounds__(G_THREADS) gemm_tc_kernel(GemmArgs a) {
   tc::fence_before();
   __syncthreads();
   if (warp == 0) tc::tmem_free(tmem, TN);
+}
+
+template <int TN, int ST>
+__global__ void __launch_bounds__(G_THREADS) gemm_tc_kernel(GemmArgs a) {
+  gemm_tile<TN, ST>(a, (int64_t)blockIdx.x * 128, blockIdx.y * TN, 0, a.K, a.D32);
+}
+
+// Several products with a long K (the weight gradients, K = rows of the batch) in one
+// launch: block (x, z) takes tile x of the list of all products' tiles over the K slice
+// z and writes its partial sums to slice z of the product's partial array; the sum over
+// the slices is sum_slices_kernel's.
+constexpr int G_GROUP = 3;
+struct GemmGroup {
+  GemmArgs g[G_GROUP];   // D32: partial array, slices M * ldd floats apart
+  int tile0[G_GROUP + 1];
+  int kslice;            // a multiple of G_KC
+};
+
+template <int TN, int ST>
+__global__ void __launch_bounds__(G_THREADS) gemm_group_kernel(const __grid_constant__ GemmGroup gg) {
+  int p = 0;
+  while (p + 1 < G_GROUP && (int)blockIdx.x >= gg.tile0[p + 1]) ++p;
+  const GemmArgs& a = gg.g[p];
+  const int t = blockIdx.x - gg.tile0[p], mt = a.M / 128;
+  const int kbeg = blockIdx.z * gg.kslice;
+  gemm_tile<TN, ST>(a, (int64_t)(t % mt) * 128, (t / mt) * TN, kbeg, min(a.K, kbeg + gg.kslice),
+                    a.D32 + (int64_t)blockIdx.z * a.M * a.ldd);
 }
 
 // out[c][r] = in[r][c] for a BF16 R x C matrix (row strides ld_in, ld_out)
@@ -188,43 +225,67 @@ __global__ void __launch_bounds__(256) transpose_bf16_kernel(const __nv_bfloat16
   }
 }
 
-// out[c] = sum over rows of in[r][c] (FP32 in, FP64 sum in a fixed order)
-__global__ void __launch_bounds__(256) colsum_kernel(const float* __restrict__ in, int64_t ld, int R, int C,
-                                                     float* __restrict__ out) {
+// Column sums of up to three FP32 matrices of the same row count, in FP64: block (x, y)
+// sums the row slice y of 32 columns of the joint column list into part[y][column]; the
+// sum over the slices is sum_slices_kernel's.
+struct ColSums {
+  const float* in[G_GROUP];
+  int C[G_GROUP];   // columns, multiples of 32
+  int c0[G_GROUP];  // first joint column
+};
+__global__ void __launch_bounds__(256) colsum_kernel(ColSums m, int rows, int rslice, int ctot,
+                                                     double* __restrict__ part) {
   __shared__ double sh[8][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int c = blockIdx.x * 32 + tx;
+  const int c = blockIdx.x * 32;
+  int p = 0;
+  while (p + 1 < G_GROUP && c >= m.c0[p + 1]) ++p;
+  const float* in = m.in[p] + (c - m.c0[p]) + tx;
+  const int r0 = blockIdx.y * rslice, r1 = min(rows, r0 + rslice);
   double acc = 0.0;
-  if (c < C)
-    for (int r = ty; r < R; r += 8) acc += (double)in[(int64_t)r * ld + c];
+#pragma unroll 4
+  for (int r = r0 + ty; r < r1; r += 8) acc += (double)in[(int64_t)r * m.C[p]];
   sh[ty][tx] = acc;
   __syncthreads();
-  if (ty == 0 && c < C) {
+  if (ty == 0) {
     double t = 0.0;
     for (int j = 0; j < 8; ++j) t += sh[j][tx];
-    out[c] = (float)t;
+    part[(int64_t)blockIdx.y * ctot + c + tx] = t;
   }
 }
 
-// dO = 2 (O - T) / (rows * nout) on the first nout columns (0 beyond), FP32 and
-// BF16; per-block partial sums of (O - T)^2 in FP64.
+// dO = 2 (O - T) / (rows * nout) on the first nout columns (0 beyond), FP32 and BF16,
+// row-major and (BF16) transposed; per-block partial sums of (O - T)^2 in FP64.  One
+// block per 32 rows of 128 columns at a time, the transpose through shared memory.
 __global__ void __launch_bounds__(256) mse_grad_kernel(const float* __restrict__ O, const float* __restrict__ T,
-                                                       int64_t rows, int ld, int nout, float* __restrict__ dO,
-                                                       __nv_bfloat16* __restrict__ dO16, double* __restrict__ part) {
+                                                       int64_t rows, int nout, float* __restrict__ dO,
+                                                       __nv_bfloat16* __restrict__ dO16,
+                                                       __nv_bfloat16* __restrict__ dO16T, double* __restrict__ part) {
   __shared__ double sh[256];
+  __shared__ __nv_bfloat16 tile[32][130];
   const double scale = 2.0 / ((double)rows * nout);
   double acc = 0.0;
-  const int64_t total = rows * ld;
-  for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < total; i += (int64_t)gridDim.x * 256) {
-    const int c = (int)(i % ld);
-    float g = 0.f;
-    if (c < nout) {
-      const float d = O[i] - T[i];
-      acc += (double)d * d;
-      g = (float)(scale * d);
+  for (int64_t r0 = (int64_t)blockIdx.x * 32; r0 < rows; r0 += (int64_t)gridDim.x * 32) {
+    for (int e = threadIdx.x; e < 32 * 128; e += 256) {
+      const int c = e & 127, r = e >> 7;
+      const int64_t i = (r0 + r) * 128 + c;
+      float g = 0.f;
+      if (c < nout) {
+        const float d = O[i] - T[i];
+        acc += (double)d * d;
+        g = (float)(scale * d);
+      }
+      dO[i] = g;
+      const __nv_bfloat16 h = __float2bfloat16(g);
+      dO16[i] = h;
+      tile[r][c] = h;
     }
-    dO[i] = g;
-    dO16[i] = __float2bfloat16(g);
+    __syncthreads();
+    for (int e = threadIdx.x; e < 32 * 128; e += 256) {
+      const int r = e & 31, c = e >> 5;
+      dO16T[(int64_t)c * rows + r0 + r] = tile[r][c];
+    }
+    __syncthreads();
   }
   sh[threadIdx.x] = acc;
   __syncthreads();
@@ -235,11 +296,55 @@ __global__ void __launch_bounds__(256) mse_grad_kernel(const float* __restrict__
   if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
-__global__ void sum_partials_kernel(const double* __restrict__ part, int n, double scale, double* __restrict__ out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
+// Sums over the slices, in slice order: the weight gradients (three FP32 partial arrays,
+// at most 16 slices) and, in the last block, the bias gradients (joint columns of
+// colsum_kernel, FP64) and the loss from its per-block parts (FP64).
+struct SliceSums {
+  const float* w[G_GROUP];
+  int64_t nw[G_GROUP];      // elements per slice
+  float* wout[G_GROUP];
+  int wslices;
+  const double* b;
+  int bslices, ctot;
+  int c0[G_GROUP];
+  float* bout[G_GROUP];
+  const double* loss_part;
+  int nloss;
+  double loss_scale;
+  double* loss;
+};
+__global__ void __launch_bounds__(256) sum_slices_kernel(const __grid_constant__ SliceSums m) {
+  if (blockIdx.x == gridDim.x - 1) {
+    __shared__ double sh[256];
     double t = 0.0;
-    for (int i = 0; i < n; ++i) t += part[i];
-    *out = t * scale;
+    for (int i = threadIdx.x; i < m.nloss; i += 256) t += m.loss_part[i];
+    sh[threadIdx.x] = t;
+    __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+      if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
+      __syncthreads();
+    }
+    if (threadIdx.x == 0) *m.loss = sh[0] * m.loss_scale;
+    for (int c = threadIdx.x; c < m.ctot; c += 256) {
+      int p = 0;
+      while (p + 1 < G_GROUP && c >= m.c0[p + 1]) ++p;
+      double v = 0.0;
+      for (int s = 0; s < m.bslices; ++s) v += m.b[(int64_t)s * m.ctot + c];
+      m.bout[p][c - m.c0[p]] = (float)v;
+    }
+    return;
+  }
+  int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+#pragma unroll
+  for (int p = 0; p < G_GROUP; ++p) {
+    if (i < m.nw[p]) {
+      float v = 0.f;
+#pragma unroll 4
+      for (int s = 0; s < m.wslices; ++s) v += m.w[p][(int64_t)s * m.nw[p] + i];
+      m.wout[p][i] = v;
+      return;
+    }
+    i -= m.nw[p];
   }
 }
 
@@ -366,19 +471,30 @@ unsigned grid_for(int64_t n, int threads, int64_t cap = 1 << 20) {
 
 }  // namespace
 
-cudaError_t launch_gemm_tc(const GemmArgs& a, cudaStream_t s, int* nl) {
+namespace {
+constexpr int G_ST = 4;  // stages of the K pipeline
+size_t gemm_smem(int TN) { return G_ST * ((size_t)G_A_BYTES + (size_t)TN * G_KC * 2 + 8) + 16; }
+bool gemm_ok(const GemmArgs& a) {
+  if (a.M % 128 || a.N % 16 || a.K % 16 || a.K <= 0 || a.lda % 8 || a.ldb % 8) return false;
+  return !((a.D32 && a.ldd % 4) || (a.D16 && a.ldd16 % 8) || (a.epi == GEMM_EPI_DGELU && (!a.Zin || a.ldz % 4)));
+}
+}  // namespace
+
+cudaError_t launch_gemm_tc(const GemmArgs& a, int num_sms, cudaStream_t s, int* nl) {
   if (a.M <= 0 || a.N <= 0) return cudaSuccess;
-  if (a.M % 128 || a.N % 16 || a.K % 16 || a.K <= 0 || a.lda % 8 || a.ldb % 8) return cudaErrorInvalidValue;
-  if ((a.D32 && a.ldd % 4) || (a.D16 && a.ldd16 % 8) || (a.epi == GEMM_EPI_DGELU && (!a.Zin || a.ldz % 4)))
-    return cudaErrorInvalidValue;
-  const int TN = a.N > 128 ? 256 : (a.N > 64 ? 128 : 64);
-  const size_t smem = 2 * ((size_t)G_A_BYTES + (size_t)TN * G_KC * 2) + 64;
+  if (!gemm_ok(a)) return cudaErrorInvalidValue;
+  // the widest tile that still gives two blocks per SM: latency (the K pipeline, then an
+  // epilogue of 40 instructions per element with GELU) is most of a block's time, so small
+  // batches want more and smaller blocks (8192 x 256 x 432 with GELU: 64 blocks of 256
+  // columns and two stages 31 us, 256 blocks of 64 columns and four stages 24 us, cold)
+  int TN = a.N > 128 ? 256 : (a.N > 64 ? 128 : 64);
+  while (TN > 64 && (int64_t)(a.M / 128) * ((a.N + TN - 1) / TN) < 2 * num_sms) TN /= 2;
   dim3 grid((unsigned)(a.M / 128), (unsigned)((a.N + TN - 1) / TN));
   cudaError_t e;
-#define GEMM_LAUNCH(T)                                                                                   \
-  e = cudaFuncSetAttribute(gemm_tc_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-  if (e != cudaSuccess) return e;                                                                       \
-  gemm_tc_kernel<T><<<grid, G_THREADS, smem, s>>>(a)
+#define GEMM_LAUNCH(T)                                                                                          \
+  e = cudaFuncSetAttribute(gemm_tc_kernel<T, G_ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(T)); \
+  if (e != cudaSuccess) return e;                                                                              \
+  gemm_tc_kernel<T, G_ST><<<grid, G_THREADS, gemm_smem(T), s>>>(a)
   if (TN == 256) {
     GEMM_LAUNCH(256);
   } else if (TN == 128) {
@@ -391,6 +507,60 @@ cudaError_t launch_gemm_tc(const GemmArgs& a, cudaStream_t s, int* nl) {
   return cudaGetLastError();
 }
 
+int weight_grad_slices(int64_t rows) { return (int)std::min<int64_t>(16, std::max<int64_t>(1, rows / 256)); }
+
+// A gradient over 8192 rows was three products of 2 to 4 blocks that walk K = 8192 alone
+// (257 us each), three column sums of at most 8 blocks (160 us each) and a one-thread
+// loss sum (36 us); split over 16 row slices: 30, 32 and 23 us in all (cold; whole
+// backward pass with its result copy 1530 -> 270 us).
+cudaError_t launch_weight_grads(const GemmArgs g[3], const float* const dz[3], const int cols[3], float* const bout[3],
+                                int rows, float* wpart, double* bpart, const double* loss_part, int nloss,
+                                double loss_scale, double* loss, cudaStream_t s, int* nl) {
+  constexpr int TN = 128;
+  const int slices = weight_grad_slices(rows);
+  GemmGroup gg;
+  SliceSums ss;
+  ColSums cs;
+  gg.tile0[0] = 0;
+  gg.kslice = (int)(((int64_t)rows / slices + G_KC - 1) / G_KC * G_KC);
+  const int used = (rows + gg.kslice - 1) / gg.kslice;
+  int64_t off = 0, nw = 0;
+  int ctot = 0;
+  for (int p = 0; p < G_GROUP; ++p) {
+    gg.g[p] = g[p];
+    if (g[p].M <= 0 || g[p].N <= 0 || g[p].K != rows || !gemm_ok(g[p]) || g[p].ldd != g[p].N || cols[p] % 32)
+      return cudaErrorInvalidValue;
+    ss.wout[p] = g[p].D32;
+    ss.nw[p] = (int64_t)g[p].M * g[p].N;
+    ss.w[p] = gg.g[p].D32 = wpart + off;
+    off += ss.nw[p] * used;
+    nw += ss.nw[p];
+    gg.tile0[p + 1] = gg.tile0[p] + g[p].M / 128 * ((g[p].N + TN - 1) / TN);
+    cs.in[p] = dz[p];
+    cs.C[p] = cols[p];
+    cs.c0[p] = ss.c0[p] = ctot;
+    ss.bout[p] = bout[p];
+    ctot += cols[p];
+  }
+  cudaError_t e = cudaFuncSetAttribute(gemm_group_kernel<TN, G_ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)gemm_smem(TN));
+  if (e != cudaSuccess) return e;
+  gemm_group_kernel<TN, G_ST><<<dim3((unsigned)gg.tile0[G_GROUP], 1, (unsigned)used), G_THREADS, gemm_smem(TN), s>>>(gg);
+  const int rslice = (rows + slices - 1) / slices;
+  colsum_kernel<<<dim3((unsigned)(ctot / 32), (unsigned)slices), 256, 0, s>>>(cs, rows, rslice, ctot, bpart);
+  ss.wslices = used;
+  ss.b = bpart;
+  ss.bslices = slices;
+  ss.ctot = ctot;
+  ss.loss_part = loss_part;
+  ss.nloss = nloss;
+  ss.loss_scale = loss_scale;
+  ss.loss = loss;
+  sum_slices_kernel<<<(unsigned)((nw + 255) / 256 + 1), 256, 0, s>>>(ss);
+  *nl += 3;
+  return cudaGetLastError();
+}
+
 cudaError_t launch_transpose_bf16(const void* in, int64_t ld_in, void* out, int64_t ld_out, int R, int C,
                                   cudaStream_t s, int* nl) {
   if (R <= 0 || C <= 0) return cudaSuccess;
@@ -400,17 +570,14 @@ cudaError_t launch_transpose_bf16(const void* in, int64_t ld_in, void* out, int6
   return cudaGetLastError();
 }
 
-cudaError_t launch_colsum(const float* in, int64_t ld, int R, int C, float* out, cudaStream_t s, int* nl) {
-  colsum_kernel<<<(unsigned)((C + 31) / 32), 256, 0, s>>>(in, ld, R, C, out);
-  ++*nl;
-  return cudaGetLastError();
-}
+int mse_grad_parts(int64_t rows) { return (int)std::min<int64_t>(512, (rows + 31) / 32); }
 
-cudaError_t launch_mse_grad(const float* O, const float* T, int64_t rows, int ld, int nout, float* dO, void* dO16,
-                            double* part, int nparts, double* loss, cudaStream_t s, int* nl) {
-  mse_grad_kernel<<<(unsigned)nparts, 256, 0, s>>>(O, T, rows, ld, nout, dO, (__nv_bfloat16*)dO16, part);
-  sum_partials_kernel<<<1, 32, 0, s>>>(part, nparts, 1.0 / ((double)rows * nout), loss);
-  *nl += 2;
+cudaError_t launch_mse_grad(const float* O, const float* T, int64_t rows, int nout, float* dO, void* dO16, void* dO16T,
+                            double* part, cudaStream_t s, int* nl) {
+  if (rows % 32) return cudaErrorInvalidValue;
+  mse_grad_kernel<<<(unsigned)mse_grad_parts(rows), 256, 0, s>>>(O, T, rows, nout, dO, (__nv_bfloat16*)dO16,
+                                                                 (__nv_bfloat16*)dO16T, part);
+  ++*nl;
   return cudaGetLastError();
 }
 

@@ -46,6 +46,8 @@ struct pmmm_surrogate {
   int64_t cap = 0;
   __nv_bfloat16 *Y1 = nullptr, *Y2 = nullptr, *dO16 = nullptr, *dZ2_16 = nullptr, *dZ1_16 = nullptr;
   __nv_bfloat16 *Xt = nullptr, *Y1t = nullptr, *Y2t = nullptr, *dOt = nullptr, *dZ2t = nullptr, *dZ1t = nullptr;
+  float* wpart = nullptr;   // K slices of the weight gradients
+  double* bpart = nullptr;  // row slices of the bias gradients
   float *Z1 = nullptr, *Z2 = nullptr, *O = nullptr, *dO = nullptr, *dZ2 = nullptr, *dZ1 = nullptr;
   __nv_bfloat16* Xc = nullptr;  // features of the evaluated system [Kp][432]
   float* Lcorr = nullptr;       // corrected locals [C_hi][K]
@@ -79,7 +81,7 @@ int ensure_ws(pmmm_surrogate* s, int64_t rows) {
   if (rows <= s->cap) return PMMM_OK;
   cudaStreamSynchronize(s->stream);
   void* old[] = {s->Y1, s->Y2, s->dO16, s->dZ2_16, s->dZ1_16, s->Xt, s->Y1t, s->Y2t, s->dOt, s->dZ2t, s->dZ1t,
-                 s->Z1, s->Z2, s->O, s->dO, s->dZ2, s->dZ1};
+                 s->Z1, s->Z2, s->O, s->dO, s->dZ2, s->dZ1, s->wpart, s->bpart};
   for (void* p : old) sfree(s, p);
   s->cap = 0;
   cudaError_t e = cudaSuccess;
@@ -101,6 +103,9 @@ int ensure_ws(pmmm_surrogate* s, int64_t rows) {
   if (e == cudaSuccess) e = salloc(s, &s->dO, R * S_OP);
   if (e == cudaSuccess) e = salloc(s, &s->dZ2, R * S_H);
   if (e == cudaSuccess) e = salloc(s, &s->dZ1, R * S_H);
+  const size_t slices = (size_t)weight_grad_slices(rows);
+  if (e == cudaSuccess) e = salloc(s, &s->wpart, slices * (size_t)NPARAM);
+  if (e == cudaSuccess) e = salloc(s, &s->bpart, slices * (size_t)(2 * S_H + S_OP));
   if (e != cudaSuccess) return plan_map_cuda(e);
   s->cap = rows;
   return PMMM_OK;
@@ -136,9 +141,11 @@ GemmArgs gemm(const __nv_bfloat16* A, int64_t lda, const __nv_bfloat16* B, int64
   return g;
 }
 
-// forward pass of `rows` feature rows X [rows][432] -> O [rows][128] (Z1, Y1, Z2, Y2 kept)
-cudaError_t forward(pmmm_surrogate* s, const __nv_bfloat16* X, int rows, int* nl) {
+// forward pass of `rows` feature rows X [rows][432] -> O [rows][128] (Z1, Y1, Z2, Y2
+// kept; for training also the transposed activations)
+cudaError_t forward(pmmm_surrogate* s, const __nv_bfloat16* X, int rows, bool train, int* nl) {
   cudaStream_t st = s->stream;
+  const int sms = s->lo->num_sms;
   SCK(refresh_bf16(s, nl));
   GemmArgs g = gemm(X, S_IN, s->W1b, S_IN, rows, S_H, S_IN);
   g.bias = s->theta + OFF_B1;
@@ -147,8 +154,10 @@ cudaError_t forward(pmmm_surrogate* s, const __nv_bfloat16* X, int rows, int* nl
   g.ldd = S_H;
   g.D16 = s->Y1;
   g.ldd16 = S_H;
+  g.D16T = train ? s->Y1t : nullptr;
+  g.ldd16t = rows;
   g.err = s->err;
-  SCK(launch_gemm_tc(g, st, nl));
+  SCK(launch_gemm_tc(g, sms, st, nl));
   g = gemm(s->Y1, S_H, s->W2b, S_H, rows, S_H, S_H);
   g.bias = s->theta + OFF_B2;
   g.epi = GEMM_EPI_GELU;
@@ -156,29 +165,25 @@ cudaError_t forward(pmmm_surrogate* s, const __nv_bfloat16* X, int rows, int* nl
   g.ldd = S_H;
   g.D16 = s->Y2;
   g.ldd16 = S_H;
+  g.D16T = train ? s->Y2t : nullptr;
+  g.ldd16t = rows;
   g.err = s->err;
-  SCK(launch_gemm_tc(g, st, nl));
+  SCK(launch_gemm_tc(g, sms, st, nl));
   g = gemm(s->Y2, S_H, s->W3b, S_H, rows, S_OP, S_H);
   g.bias = s->theta + OFF_B3;
   g.D32 = s->O;
   g.ldd = S_OP;
   g.err = s->err;
-  return launch_gemm_tc(g, st, nl);
+  return launch_gemm_tc(g, sms, st, nl);
 }
 
-// gradients of the mean-squared error of the last forward pass against T into s->grad
+// gradients of the mean-squared error of the last (training) forward pass against T into s->grad
 cudaError_t backward(pmmm_surrogate* s, const __nv_bfloat16* X, const float* T, int rows, int* nl) {
   cudaStream_t st = s->stream;
-  SCK(launch_mse_grad(s->O, T, rows, S_OP, s->C_hi, s->dO, s->dO16, s->part, LOSS_PARTS, s->loss_d, st, nl));
-  SCK(launch_colsum(s->dO, S_OP, rows, S_OP, s->grad + OFF_B3, st, nl));
-  SCK(launch_transpose_bf16(s->dO16, S_OP, s->dOt, rows, rows, S_OP, st, nl));
-  SCK(launch_transpose_bf16(s->Y2, S_H, s->Y2t, rows, rows, S_H, st, nl));
-  GemmArgs g = gemm(s->dOt, rows, s->Y2t, rows, S_OP, S_H, rows);  // dW3 = dO^T Y2
-  g.D32 = s->grad + OFF_W3;
-  g.ldd = S_H;
-  g.err = s->err;
-  SCK(launch_gemm_tc(g, st, nl));
-  g = gemm(s->dO16, S_OP, s->W3t, S_OP, rows, S_H, S_OP);  // dZ2 = (dO W3) * gelu'(Z2)
+  const int sms = s->lo->num_sms;
+  SCK(launch_transpose_bf16(X, S_IN, s->Xt, rows, rows, S_IN, st, nl));
+  SCK(launch_mse_grad(s->O, T, rows, s->C_hi, s->dO, s->dO16, s->dOt, s->part, st, nl));
+  GemmArgs g = gemm(s->dO16, S_OP, s->W3t, S_OP, rows, S_H, S_OP);  // dZ2 = (dO W3) * gelu'(Z2)
   g.epi = GEMM_EPI_DGELU;
   g.Zin = s->Z2;
   g.ldz = S_H;
@@ -186,16 +191,10 @@ cudaError_t backward(pmmm_surrogate* s, const __nv_bfloat16* X, const float* T, 
   g.ldd = S_H;
   g.D16 = s->dZ2_16;
   g.ldd16 = S_H;
+  g.D16T = s->dZ2t;
+  g.ldd16t = rows;
   g.err = s->err;
-  SCK(launch_gemm_tc(g, st, nl));
-  SCK(launch_colsum(s->dZ2, S_H, rows, S_H, s->grad + OFF_B2, st, nl));
-  SCK(launch_transpose_bf16(s->dZ2_16, S_H, s->dZ2t, rows, rows, S_H, st, nl));
-  SCK(launch_transpose_bf16(s->Y1, S_H, s->Y1t, rows, rows, S_H, st, nl));
-  g = gemm(s->dZ2t, rows, s->Y1t, rows, S_H, S_H, rows);  // dW2 = dZ2^T Y1
-  g.D32 = s->grad + OFF_W2;
-  g.ldd = S_H;
-  g.err = s->err;
-  SCK(launch_gemm_tc(g, st, nl));
+  SCK(launch_gemm_tc(g, sms, st, nl));
   g = gemm(s->dZ2_16, S_H, s->W2t, S_H, rows, S_H, S_H);  // dZ1 = (dZ2 W2) * gelu'(Z1)
   g.epi = GEMM_EPI_DGELU;
   g.Zin = s->Z1;
@@ -204,16 +203,25 @@ cudaError_t backward(pmmm_surrogate* s, const __nv_bfloat16* X, const float* T, 
   g.ldd = S_H;
   g.D16 = s->dZ1_16;
   g.ldd16 = S_H;
+  g.D16T = s->dZ1t;
+  g.ldd16t = rows;
   g.err = s->err;
-  SCK(launch_gemm_tc(g, st, nl));
-  SCK(launch_colsum(s->dZ1, S_H, rows, S_H, s->grad + OFF_B1, st, nl));
-  SCK(launch_transpose_bf16(s->dZ1_16, S_H, s->dZ1t, rows, rows, S_H, st, nl));
-  SCK(launch_transpose_bf16(X, S_IN, s->Xt, rows, rows, S_IN, st, nl));
-  g = gemm(s->dZ1t, rows, s->Xt, rows, S_H, S_IN, rows);  // dW1 = dZ1^T X
-  g.D32 = s->grad + OFF_W1;
-  g.ldd = S_IN;
-  g.err = s->err;
-  return launch_gemm_tc(g, st, nl);
+  SCK(launch_gemm_tc(g, sms, st, nl));
+  // dW1 = dZ1^T X, dW2 = dZ2^T Y1, dW3 = dO^T Y2; biases: the column sums of dZ1, dZ2, dO
+  GemmArgs w[3] = {gemm(s->dZ1t, rows, s->Xt, rows, S_H, S_IN, rows), gemm(s->dZ2t, rows, s->Y1t, rows, S_H, S_H, rows),
+                   gemm(s->dOt, rows, s->Y2t, rows, S_OP, S_H, rows)};
+  w[0].D32 = s->grad + OFF_W1;
+  w[0].ldd = S_IN;
+  w[1].D32 = s->grad + OFF_W2;
+  w[1].ldd = S_H;
+  w[2].D32 = s->grad + OFF_W3;
+  w[2].ldd = S_H;
+  for (GemmArgs& x : w) x.err = s->err;
+  const float* dz[3] = {s->dZ1, s->dZ2, s->dO};
+  const int cols[3] = {S_H, S_H, S_OP};
+  float* bout[3] = {s->grad + OFF_B1, s->grad + OFF_B2, s->grad + OFF_B3};
+  return launch_weight_grads(w, dz, cols, bout, rows, s->wpart, s->bpart, s->part, mse_grad_parts(rows),
+                             1.0 / ((double)rows * s->C_hi), s->loss_d, st, nl);
 }
 
 void free_sur(pmmm_surrogate* s) {
@@ -408,7 +416,7 @@ int pmmm_surrogate_forward(pmmm_surrogate* s, const void* X, int64_t rows, float
   int rc = ensure_ws(s, rows);
   if (rc != PMMM_OK) return rc;
   int nl = 0;
-  cudaError_t e = forward(s, (const __nv_bfloat16*)X, (int)rows, &nl);
+  cudaError_t e = forward(s, (const __nv_bfloat16*)X, (int)rows, false, &nl);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(out, s->O, sizeof(float) * (size_t)rows * S_OP, cudaMemcpyDeviceToDevice, s->stream);
   return status_of(s, e);
@@ -420,7 +428,7 @@ int pmmm_surrogate_gradients(pmmm_surrogate* s, const void* X, const float* T, i
   int rc = ensure_ws(s, rows);
   if (rc != PMMM_OK) return rc;
   int nl = 0;
-  cudaError_t e = forward(s, (const __nv_bfloat16*)X, (int)rows, &nl);
+  cudaError_t e = forward(s, (const __nv_bfloat16*)X, (int)rows, true, &nl);
   if (e == cudaSuccess) e = backward(s, (const __nv_bfloat16*)X, T, (int)rows, &nl);
   if (e == cudaSuccess && grad_host)
     e = cudaMemcpyAsync(grad_host, s->grad, sizeof(float) * NPARAM, cudaMemcpyDeviceToHost, s->stream);
@@ -433,7 +441,7 @@ int pmmm_surrogate_train_step(pmmm_surrogate* s, const void* X, const float* T, 
   int rc = ensure_ws(s, rows);
   if (rc != PMMM_OK) return rc;
   int nl = 0;
-  cudaError_t e = forward(s, (const __nv_bfloat16*)X, (int)rows, &nl);
+  cudaError_t e = forward(s, (const __nv_bfloat16*)X, (int)rows, true, &nl);
   if (e == cudaSuccess) e = backward(s, (const __nv_bfloat16*)X, T, (int)rows, &nl);
   if (e == cudaSuccess) e = launch_adam(s->theta, s->grad, s->am, s->av, NPARAM, lr, s->step + 1, s->stream, &nl);
   if (e != cudaSuccess) return plan_map_cuda(e);
@@ -454,7 +462,7 @@ int pmmm_surrogate_compute(pmmm_surrogate* s, int64_t n, const void* pos, const 
   s->hook.fn = [s, nmesh](cudaStream_t st, int* nl) -> cudaError_t {
     SCK(launch_gather_features((const float*)s->lo->M, s->K, nmesh, s->lo->g.periodic, s->in_scale, s->Xc, S_IN, st,
                                nl));
-    SCK(forward(s, s->Xc, (int)s->Kp, nl));
+    SCK(forward(s, s->Xc, (int)s->Kp, false, nl));
     return launch_combine_locals((const float*)s->lo->L, s->O, S_OP, s->K, s->C_hi, s->C_lo, s->out_scale, s->Lcorr,
                                  st, nl);
   };
