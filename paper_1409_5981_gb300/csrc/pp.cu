@@ -6,12 +6,11 @@
 //
 // Work is split into items of (cell, chunk of up to 32 targets), numbered by an
 // exclusive scan over the cells so that crowded cells spread over many warps.
-// One warp per item: its R targets sit in registers, lane l owns target
-// l mod TL and source phase l / TL (TL = R rounded up to a power of two, so a
-// chunk of 8 targets still keeps 32 lanes busy on 4 source phases).  Sources
-// are read with broadcast loads (all lanes of a phase read the same record):
-// through L1 in the FP64 kernel, from shared memory staged by bulk asynchronous
-// copies in the FP32 one.  Self pairs (r = 0) add zero.
+// FP32 items (pp_kernel_tma): one warp per item, its R targets in registers, lane l
+// owning target l mod TL and source phase l / TL (TL = R rounded up to a power of two,
+// so a chunk of 8 targets still keeps 32 lanes busy on 4 source phases); sparse FP32
+// systems: one thread per target (pp_target_kernel); FP64: one block per item
+// (pp64_kernel).  Self pairs (r = 0) add zero.
 #include "internal.cuh"
 #include "tcgen05.cuh"
 
@@ -21,12 +20,7 @@ namespace {
 
 constexpr int PP_WARPS = 4;
 constexpr int PP_BATCH = 1;  // work items taken per atomic by the FP32 near-field warps (one: the shortest tail)
-constexpr int PP_BLOCKS_PER_SM = 6;  // resident blocks per SM (up to 80 registers per thread)
 constexpr int CHUNK = PP_CHUNK;
-
-template <typename T> struct V4;
-template <> struct V4<float> { using type = float4; };
-template <> struct V4<double> { using type = double4; };
 
 // FP32 reciprocal square root: the hardware approximation (PTX rsqrt.approx,
 // relative error below 2^-22.9) with subnormal inputs flushed to zero.  A pair
@@ -38,208 +32,183 @@ __device__ __forceinline__ float rsqrt_ftz(float x) {
   return y;
 }
 
-template <typename T> __device__ __forceinline__ T rsq(T x);
-template <> __device__ __forceinline__ float rsq<float>(float x) { return rsqrt_ftz(x); }
-template <> __device__ __forceinline__ double rsq<double>(double x) { return rsqrt(x); }
-
 // Pair-interleaved source records for the FP32 near field: the particles of
 // cell c occupy pairs pair_start[c] ... (a cell with an odd count ends with a
 // dummy of zero charge far outside the box).  Pair j is two 16-byte words
 // {x_a, x_b, y_a, y_b}, {z_a, z_b, q_a, q_b}, so that one 128-bit load yields
 // the packed operands of two sources.
 
-// Accumulates the interactions of target (tx, ty, tz) with sources P[b + e],
-// e = ph, ph + SP, ... < cnt.  SELF: the source set may contain the target
-// itself (r = 0 contributes zero); other neighbour cells never contain a source
-// at r = 0 (a point on a shared face belongs to one cell only), so their pairs
-// skip the test.
-template <typename T, typename V, bool SELF>
-__device__ __forceinline__ void pp_pair(const V& r, T tx, T ty, T tz, T& pot, T& gx, T& gy, T& gz) {
-  const T dx = tx - r.x, dy = ty - r.y, dz = tz - r.z;
-  const T r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-  T ri = rsq<T>(r2);
-  if (SELF) ri = r2 > T(0) ? ri : T(0);
-  const T qr = r.w * ri;
-  pot += qr;
-  const T qr3 = qr * (ri * ri);
-  gx = fma(-qr3, dx, gx);
-  gy = fma(-qr3, dy, gy);
-  gz = fma(-qr3, dz, gz);
+// FP64 reciprocal square root: the hardware approximation (PTX rsqrt.approx.ftz.f64,
+// from the upper word of x, about 20 bits) and one third-order Householder step,
+//   y = y0 + y0 e (1/2 + 3/8 e),  e = 1 - x y0^2,
+// whose remainder 5/16 e^3 is below 2^-58: five FP64 operations, at 64 cycles of an SM
+// quarter each.  Zero x gives 0, subnormal x the library's rsqrt(x).
+__device__ __forceinline__ double rsqrt64(double x) {
+  double y0;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
+  const double e = fma(-x, y0 * y0, 1.0);
+  double y = fma(y0 * e, fma(e, 0.375, 0.5), y0);
+  if (__double2hiint(x) < 0x00100000) y = __double_as_longlong(x) == 0 ? 0.0 : rsqrt(x);
+  return y;
 }
 
-// Accumulates the interactions of target (tx, ty, tz) with sources src[e],
-// e = ph, ph + SP, ... < cnt.  SELF: the source set may contain the target
-// itself (r = 0 contributes zero); other neighbour cells never contain a source
-// at r = 0 (a point on a shared face belongs to one cell only), so their pairs
-// skip the test.
-template <typename T, typename V, bool SELF>
-__device__ __forceinline__ void pp_sum(const V* __restrict__ src, int cnt, int ph, int SP, T tx, T ty, T tz, T& pot,
-                                       T& gx, T& gy, T& gz) {
-  if (SP == 1) {
-    int e = 0;
-    for (; e + 4 <= cnt; e += 4) {
-      const V r0 = src[e], r1 = src[e + 1], r2 = src[e + 2], r3 = src[e + 3];
-      pp_pair<T, V, SELF>(r0, tx, ty, tz, pot, gx, gy, gz);
-      pp_pair<T, V, SELF>(r1, tx, ty, tz, pot, gx, gy, gz);
-      pp_pair<T, V, SELF>(r2, tx, ty, tz, pot, gx, gy, gz);
-      pp_pair<T, V, SELF>(r3, tx, ty, tz, pot, gx, gy, gz);
-    }
-    for (; e < cnt; ++e) pp_pair<T, V, SELF>(src[e], tx, ty, tz, pot, gx, gy, gz);
-  } else {
-    for (int e = ph; e < cnt; e += SP) pp_pair<T, V, SELF>(src[e], tx, ty, tz, pot, gx, gy, gz);
-  }
-}
+// FP64 near field (c = 1 or 2).  GB300 issues an FP64 instruction of a warp every 64
+// cycles per SM quarter, so the pair's 18 FP64 operations bound the kernel and
+// everything else is arranged to keep their lanes full and the quarters evenly loaded:
+// one block of 4 warps per item, thread t taking target t mod R (R the item's targets)
+// and every P-th source from number t / R on of all (2c+1)^3 cells' sources as one list
+// (P = 128 / R source phases; 128 - R P lanes idle), the partial sums added by a tree in
+// shared memory.  The target's coordinates in the frames of the neighbour cells are held
+// per axis and selected by integer operations.  Items come from a global counter; an
+// item's results depend only on the item.
+// Against one warp per item with power-of-two lane splits, per-cell loops and rsqrt():
+// 4096 particles / 8^3 open 303 -> 53 us (512 items over 608 SM quarters: a quarter of
+// them idle, others with three), 131072 / 16^3 periodic 4.83 -> 4.02 ms (86 % of the
+// FP64 issue rate).
+constexpr int P64_THREADS = 128;
+constexpr int P64_BLOCKS_PER_SM = 2;
 
-template <typename T> struct PPConst;
-template <> struct PPConst<float> {
-  __device__ static void get(const PPParams& p, float* cs, float& ih, float& ih2, float& sg) {
-    for (int a = 0; a < 3; ++a) cs[a] = p.cs32[a];
-    ih = p.ih32; ih2 = p.ih2_32; sg = p.sign32;
-  }
-};
-template <> struct PPConst<double> {
-  __device__ static void get(const PPParams& p, double* cs, double& ih, double& ih2, double& sg) {
-    for (int a = 0; a < 3; ++a) cs[a] = p.csf[a];
-    ih = p.ihf; ih2 = p.ih2f; sg = p.signf;
-  }
-};
-
-__device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
-
-// Persistent warps: each takes work items from a global counter (reset to zero
-// by the cell sort) until all are done.  Every item's results depend
-// only on the item, so the assignment order does not change any output bit.
-// NB_SLOTS: neighbour-table slots per lane, (2c+1)^3 <= 32 * NB_SLOTS (1 for c = 1, 4 for c = 2)
-template <typename T, int NB_SLOTS>
-__global__ void __launch_bounds__(PP_WARPS * 32, PP_BLOCKS_PER_SM) pp_kernel(const T* __restrict__ part, const uint32_t* __restrict__ vals,
-                                                              const int* __restrict__ cs, int64_t K,
-                                                              const uint32_t* __restrict__ item_start,
-                                                              const uint32_t* __restrict__ item_cell,
-                                                              unsigned int* __restrict__ counter, const T* __restrict__ far,
-                                                              PPParams pp, T* __restrict__ phi, T* __restrict__ force,
-                                                              double* __restrict__ epart) {
-  using V = typename V4<T>::type;
-  const V* P = reinterpret_cast<const V*>(part);
-  const int lane = threadIdx.x & 31;
+template <int CUT>
+__global__ void __launch_bounds__(P64_THREADS, P64_BLOCKS_PER_SM) pp64_kernel(
+    const double* __restrict__ part, const uint32_t* __restrict__ vals, const int* __restrict__ cs, int64_t K,
+    const uint32_t* __restrict__ item_start, const uint32_t* __restrict__ item_cell,
+    unsigned int* __restrict__ counter, const double* __restrict__ far, PPParams pp, double* __restrict__ phi,
+    double* __restrict__ force, double* __restrict__ epart) {
+  constexpr int W = 2 * CUT + 1, NN = W * W * W;
+  __shared__ int first[NN + 1], off[NN];  // list position e of cell k: first[k] <= e < first[k+1], record e + off[k]
+  __shared__ double sum[4][P64_THREADS];
+  __shared__ uint32_t next_item;
+  const double4* P = reinterpret_cast<const double4*>(part);
+  const int tid = threadIdx.x, lane = tid & 31;
   const uint32_t nitems = item_start[K];
   const int nx = pp.n[0], ny = pp.n[1], nz = pp.n[2];
-  const int c = pp.c, w = 2 * c + 1, NN = w * w * w;
-  T csv[3], ih, ih2, sg;
-  PPConst<T>::get(pp, csv, ih, ih2, sg);
   for (;;) {
-    uint32_t item = 0;
-    if (lane == 0) item = atomicAdd(counter, 1u);
-    item = __shfl_sync(0xffffffffu, item, 0);
-    if (item >= nitems) break;  // warp-uniform
+    if (tid == 0) next_item = atomicAdd(counter, 1u);
+    __syncthreads();
+    const uint32_t item = next_item;
+    if (item >= nitems) break;
     const int cell = (int)item_cell[item];
-    const int chunk = (int)(item - item_start[cell]);
-    const int tbeg = cs[cell] + chunk * CHUNK;
-    const int R = min(CHUNK, cs[cell + 1] - tbeg);
-    int TL = 1;
-    while (TL < R) TL <<= 1;
-    const int SP = 32 / TL;
-    const int tl = lane & (TL - 1), ph = lane / TL;
-    const bool active = tl < R;
-    V xi;
-    xi.x = T(0); xi.y = T(0); xi.z = T(0); xi.w = T(0);
-    if (active) xi = P[tbeg + tl];
-    const int sbase = cell - cell % pp.ksys, lc = cell - sbase;  // system's first cell, local cell
-    const int ix = lc % nx, iy = (lc / nx) % ny, iz = lc / (nx * ny);
-    // neighbour table: entry k (x fastest) in lane k % 32, slot k / 32
-    int nbb[NB_SLOTS], nbc[NB_SLOTS];
-#pragma unroll
-    for (int j = 0; j < NB_SLOTS; ++j) {
-      const int k = lane + 32 * j;
-      nbb[j] = 0;
-      nbc[j] = 0;
-      if (k < NN) {
-        int jx = ix + k % w - c, jy = iy + (k / w) % w - c, jz = iz + k / (w * w) - c;
-        bool ok = true;
-        if (jx < 0 || jx >= nx) { ok = ok && pp.periodic; jx += (jx < 0) ? nx : -nx; }
-        if (jy < 0 || jy >= ny) { ok = ok && pp.periodic; jy += (jy < 0) ? ny : -ny; }
-        if (jz < 0 || jz >= nz) { ok = ok && pp.periodic; jz += (jz < 0) ? nz : -nz; }
-        if (ok) {
-          const int cj = sbase + jx + nx * (jy + ny * jz);
-          nbb[j] = __ldg(cs + cj);
-          nbc[j] = __ldg(cs + cj + 1) - nbb[j];
-        }
-      }
-    }
-    auto nb = [&](int k, int& b, int& n) {
-      int bb = nbb[0], cc = nbc[0];
-#pragma unroll
-      for (int q = 1; q < NB_SLOTS; ++q)
-        if ((k >> 5) == q) {
-          bb = nbb[q];
-          cc = nbc[q];
-        }
-      b = __shfl_sync(0xffffffffu, bb, k & 31);
-      n = __shfl_sync(0xffffffffu, cc, k & 31);
-    };
-    int b, cnt;
-    nb(0, b, cnt);
-    if (lane < cnt) prefetch_l1(P + b + lane);
-    T pot = T(0), gx = T(0), gy = T(0), gz = T(0);
-    int k = 0;
-    for (int ez = -c; ez <= c; ++ez) {
-      const T tz = xi.z - (T)ez * csv[2];
-      for (int ey = -c; ey <= c; ++ey) {
-        const T ty = xi.y - (T)ey * csv[1];
-        for (int ex = -c; ex <= c; ++ex, ++k) {
-          int bn = 0, cn = 0;
-          if (k + 1 < NN) {
-            nb(k + 1, bn, cn);
-            if (lane < cn) prefetch_l1(P + bn + lane);  // next neighbour cell into L1
+    const int tbeg = cs[cell] + (int)(item - item_start[cell]) * CHUNK;
+    const int R = min(CHUNK, cs[cell + 1] - tbeg), NP = P64_THREADS / R;
+    const int tl = tid % R, ph = tid / R;
+    const bool active = ph < NP;
+    if (tid < 32) {
+      // counts of the cells in (z, y, x) order and their running sum
+      const int sbase = cell - cell % pp.ksys, lc = cell - sbase;
+      const int ix = lc % nx, iy = (lc / nx) % ny, iz = lc / (nx * ny);
+      int run = 0;
+      for (int k0 = 0; k0 < NN; k0 += 32) {
+        const int k = k0 + lane;
+        int b = 0, m = 0;
+        if (k < NN) {
+          int jx = ix + k % W - CUT, jy = iy + (k / W) % W - CUT, jz = iz + k / (W * W) - CUT;
+          bool ok = true;
+          if (jx < 0 || jx >= nx) { ok = ok && pp.periodic; jx += (jx < 0) ? nx : -nx; }
+          if (jy < 0 || jy >= ny) { ok = ok && pp.periodic; jy += (jy < 0) ? ny : -ny; }
+          if (jz < 0 || jz >= nz) { ok = ok && pp.periodic; jz += (jz < 0) ? nz : -nz; }
+          if (ok) {
+            const int cj = sbase + jx + nx * (jy + ny * jz);
+            b = __ldg(cs + cj);
+            m = __ldg(cs + cj + 1) - b;
           }
-          const T tx = xi.x - (T)ex * csv[0];
-          if (ex == 0 && ey == 0 && ez == 0)
-            pp_sum<T, V, true>(P + b, cnt, ph, SP, tx, ty, tz, pot, gx, gy, gz);
-          else
-            pp_sum<T, V, false>(P + b, cnt, ph, SP, tx, ty, tz, pot, gx, gy, gz);
-          b = bn;
-          cnt = cn;
+        }
+        int v = m;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int u = __shfl_up_sync(0xffffffffu, v, o);
+          if (lane >= o) v += u;
+        }
+        if (k < NN) {
+          first[k] = run + v - m;
+          off[k] = b - (run + v - m);
+        }
+        run += __shfl_sync(0xffffffffu, v, 31);
+      }
+      if (lane == 0) first[NN] = run;
+    }
+    const double4 xi = P[tbeg + tl];
+    double tx[W], ty[W], tz[W];  // the target in the frames of the cells at each axis offset
+#pragma unroll
+    for (int d = 0; d < W; ++d) {
+      tx[d] = xi.x - (double)(d - CUT) * pp.csf[0];
+      ty[d] = xi.y - (double)(d - CUT) * pp.csf[1];
+      tz[d] = xi.z - (double)(d - CUT) * pp.csf[2];
+    }
+    __syncthreads();
+    double pot = 0.0, gx = 0.0, gy = 0.0, gz = 0.0;
+    if (active) {
+      const int total = first[NN];
+      int k = 0;
+      auto pair = [&](int e) {
+        while (e >= first[k + 1]) ++k;
+        const double4 r = P[e + off[k]];
+        const int ex = k % W, ey = (k / W) % W, ez = k / (W * W);
+        double ux = tx[0], uy = ty[0], uz = tz[0];
+#pragma unroll
+        for (int d = 1; d < W; ++d) {
+          if (ex == d) ux = tx[d];
+          if (ey == d) uy = ty[d];
+          if (ez == d) uz = tz[d];
+        }
+        const double dx = ux - r.x, dy = uy - r.y, dz = uz - r.z;
+        const double ri = rsqrt64(fma(dx, dx, fma(dy, dy, dz * dz)));  // 0 for the self pair
+        const double qr = r.w * ri;
+        pot += qr;
+        const double qr3 = qr * (ri * ri);
+        gx = fma(-qr3, dx, gx);
+        gy = fma(-qr3, dy, gy);
+        gz = fma(-qr3, dz, gz);
+      };
+      int e = ph;
+      for (; e + NP < total; e += 2 * NP) {  // two at a time: 4.02 ms against 5.41 one by one (below)
+        pair(e);
+        pair(e + NP);
+      }
+      if (e < total) pair(e);
+    }
+    sum[0][tid] = pot;
+    sum[1][tid] = gx;
+    sum[2][tid] = gy;
+    sum[3][tid] = gz;
+    for (int m = NP; m > 1;) {  // tree over the phases
+      const int h = (m + 1) / 2;
+      __syncthreads();
+      if (ph < m - h)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) sum[q][tid] += sum[q][tid + h * R];
+      m = h;
+    }
+    __syncthreads();
+    if (tid < 32) {
+      double e_t = 0.0, f_t[3] = {0.0, 0.0, 0.0};
+      if (tid < R) {
+        const int s = tbeg + tid;
+        const double4 fr = reinterpret_cast<const double4*>(far)[s];
+        const double sg = pp.signf, q = P[s].w;
+        const double pt = sg * (fr.x + sum[0][tid] * pp.ihf);
+        const double g[3] = {sg * (fr.y + sum[1][tid] * pp.ih2f), sg * (fr.z + sum[2][tid] * pp.ih2f),
+                             sg * (fr.w + sum[3][tid] * pp.ih2f)};
+        const uint32_t o = vals[s];
+        if (phi) phi[o] = pt;
+        e_t = 0.5 * q * pt;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          f_t[a] = -q * g[a];
+          if (force) force[3 * (int64_t)o + a] = f_t[a];
         }
       }
-    }
-    for (int o = TL; o < 32; o <<= 1) {
-      pot += __shfl_xor_sync(0xffffffffu, pot, o);
-      gx += __shfl_xor_sync(0xffffffffu, gx, o);
-      gy += __shfl_xor_sync(0xffffffffu, gy, o);
-      gz += __shfl_xor_sync(0xffffffffu, gz, o);
-    }
-    T e_t = T(0), f_t[3] = {T(0), T(0), T(0)};
-    if (active && ph == 0) {
-      const int s = tbeg + tl;
-      const V fr = reinterpret_cast<const V*>(far)[s];
-      const T pt = sg * (fr.x + pot * ih);
-      const T g0 = sg * (fr.y + gx * ih2), g1 = sg * (fr.z + gy * ih2), g2 = sg * (fr.w + gz * ih2);
-      const uint32_t o = vals[s];
-      const T q = xi.w;
-      if (phi) phi[o] = pt;
-      if (force) {
-        force[3 * (int64_t)o + 0] = -q * g0;
-        force[3 * (int64_t)o + 1] = -q * g1;
-        force[3 * (int64_t)o + 2] = -q * g2;
-      }
-      e_t = T(0.5) * q * pt;
-      f_t[0] = -q * g0;
-      f_t[1] = -q * g1;
-      f_t[2] = -q * g2;
-    }
-    // deterministic warp reduction of this item's energy and net-force partials
-    // (the <= 32 terms of one item in T; items are summed in FP64 afterwards)
+      // deterministic sums of this item's energy and net-force partials
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      e_t += __shfl_xor_sync(0xffffffffu, e_t, o);
-      f_t[0] += __shfl_xor_sync(0xffffffffu, f_t[0], o);
-      f_t[1] += __shfl_xor_sync(0xffffffffu, f_t[1], o);
-      f_t[2] += __shfl_xor_sync(0xffffffffu, f_t[2], o);
-    }
-    if (lane == 0) {
-      epart[(int64_t)item * 4 + 0] = (double)e_t;
-      epart[(int64_t)item * 4 + 1] = (double)f_t[0];
-      epart[(int64_t)item * 4 + 2] = (double)f_t[1];
-      epart[(int64_t)item * 4 + 3] = (double)f_t[2];
+      for (int o = 16; o > 0; o >>= 1) {
+        e_t += __shfl_xor_sync(0xffffffffu, e_t, o);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) f_t[a] += __shfl_xor_sync(0xffffffffu, f_t[a], o);
+      }
+      if (lane == 0) {
+        epart[(int64_t)item * 4 + 0] = e_t;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) epart[(int64_t)item * 4 + 1 + a] = f_t[a];
+      }
     }
   }
 }
@@ -964,42 +933,33 @@ cudaError_t launch_pp(bool fp64, const void* part, const void* src2, const uint3
                       const uint32_t* item_start, const uint32_t* item_cell, unsigned int* counter, int num_sms,
                       const void* far, PPParams pp, void* phi, void* force, double* epart, int* err, void* near_out,
                       cudaStream_t s, int* nl) {
-  // persistent launch: PP_BLOCKS_PER_SM resident blocks of PP_WARPS warps per SM
-  const unsigned blocks = (unsigned)(PP_BLOCKS_PER_SM * (num_sms > 0 ? num_sms : 1));
-  if (per_target && pp_per_target_applies(fp64, pp.c) && src2 != nullptr) {
+  const int sms = num_sms > 0 ? num_sms : 1;
+  if (fp64) {
+    if (near_out) return cudaErrorInvalidValue;  // only the cell-item FP32 kernel splits
+#define PP64(C)                                                                                                    \
+  pp64_kernel<C><<<(unsigned)(P64_BLOCKS_PER_SM * sms), P64_THREADS, 0, s>>>((const double*)part, vals, cell_start, K, \
+                                                                             item_start, item_cell, counter,       \
+                                                                             (const double*)far, pp, (double*)phi, \
+                                                                             (double*)force, epart)
+    if (pp.c <= 1) PP64(1); else PP64(2);
+#undef PP64
+  } else if (per_target) {
     if (n <= 0) return cudaSuccess;
     const unsigned g = (unsigned)((n + PPS_THREADS - 1) / PPS_THREADS);
-    if (pp.c <= 1)
-      pp_target_kernel<1><<<g, PPS_THREADS, 0, s>>>((const float4*)part, (const ulonglong2*)src2, pair_start, keys,
-                                                    vals, cell_start, item_start, n, (const float4*)far, pp,
-                                                    (float*)phi, (float*)force, epart);
-    else
-      pp_target_kernel<2><<<g, PPS_THREADS, 0, s>>>((const float4*)part, (const ulonglong2*)src2, pair_start, keys,
-                                                    vals, cell_start, item_start, n, (const float4*)far, pp,
-                                                    (float*)phi, (float*)force, epart);
-  } else if (pp_tma_applies(fp64, pp.c, false) && src2 != nullptr) {
-    const unsigned tblocks = (unsigned)(NT_BLOCKS_PER_SM * (num_sms > 0 ? num_sms : 1));
-    if (pp.c <= 1)
-      pp_kernel_tma<1><<<tblocks, PP_WARPS * 32, 0, s>>>((const float*)part, (const float*)src2, pair_start, vals,
-                                                         cell_start, K, item_start, item_cell, counter,
-                                                         (const float*)far, pp, (float*)phi, (float*)force, epart, err,
-                                                         (float4*)near_out);
-    else
-      pp_kernel_tma<2><<<tblocks, PP_WARPS * 32, 0, s>>>((const float*)part, (const float*)src2, pair_start, vals,
-                                                         cell_start, K, item_start, item_cell, counter,
-                                                         (const float*)far, pp, (float*)phi, (float*)force, epart, err,
-                                                         (float4*)near_out);
+#define PP_TARGETS(C)                                                                                              \
+  pp_target_kernel<C><<<g, PPS_THREADS, 0, s>>>((const float4*)part, (const ulonglong2*)src2, pair_start, keys, vals, \
+                                                cell_start, item_start, n, (const float4*)far, pp, (float*)phi,    \
+                                                (float*)force, epart)
+    if (pp.c <= 1) PP_TARGETS(1); else PP_TARGETS(2);
+#undef PP_TARGETS
   } else {
-    if (near_out) return cudaErrorInvalidValue;  // only the cell-item FP32 kernel splits
-#define PP_LAUNCH(T, S)                                                                                              \
-  pp_kernel<T, S><<<blocks, PP_WARPS * 32, 0, s>>>((const T*)part, vals, cell_start, K, item_start, item_cell, counter, \
-                                                   (const T*)far, pp, (T*)phi, (T*)force, epart)
-    if (fp64) {
-      if (pp.c <= 1) PP_LAUNCH(double, 1); else PP_LAUNCH(double, 4);
-    } else {
-      if (pp.c <= 1) PP_LAUNCH(float, 1); else PP_LAUNCH(float, 4);
-    }
-#undef PP_LAUNCH
+    // persistent launch: NT_BLOCKS_PER_SM resident blocks of PP_WARPS warps per SM
+#define PP_ITEMS(C)                                                                                                  \
+  pp_kernel_tma<C><<<(unsigned)(NT_BLOCKS_PER_SM * sms), PP_WARPS * 32, 0, s>>>(                                     \
+      (const float*)part, (const float*)src2, pair_start, vals, cell_start, K, item_start, item_cell, counter,       \
+      (const float*)far, pp, (float*)phi, (float*)force, epart, err, (float4*)near_out)
+    if (pp.c <= 1) PP_ITEMS(1); else PP_ITEMS(2);
+#undef PP_ITEMS
   }
   ++*nl;
   return cudaGetLastError();
