@@ -401,7 +401,7 @@ cudaError_t mesh_stage(pmmm_plan* pl, int B, int* nl) {
     // specM -> specL (transposed) -> M2L -> specM -> specL (channel-major)
     e = launch_transpose(fp64, pl->specM, pl->specL, R, pl->d.Kh, s, nl);
     if (e == cudaSuccess)
-      e = pl->m2l_tc ? launch_m2l_tc(pl->specL, pl->G, pl->specM, pl->m2l_tab_tc, pl->p, B, pl->d.Kh, pl->num_sms,
+      e = pl->m2l_tc ? launch_m2l_tc(pl->specL, pl->Gr, pl->specM, pl->m2l_tab_tc, pl->p, B, pl->d.Kh, pl->num_sms,
                                      pl->m2l_tile, pl->err, s, nl)
                      : launch_m2l_batched(fp64, pl->specL, pl->G, pl->specM, pl->m2l_tab, pl->p, B, pl->d.Kh, s, nl);
     if (e == cudaSuccess) e = launch_transpose(fp64, pl->specM, pl->specL, pl->d.Kh, R, s, nl);
@@ -444,7 +444,7 @@ cudaError_t hier_stage(pmmm_plan* pl, int* nl) {
   if (!h.wavemajor)
     e = launch_m2l_systems(pl->p, fp64, pl->hspecM, bp->G, bp->Gr, pl->hspecL, Khh, (int)Kc, s, nl);
   else if (pl->m2l_tc)
-    e = launch_m2l_tc(pl->hspecM, bp->G, pl->hspecL, pl->m2l_tab_tc, pl->p, (int)Kc, Khh, pl->num_sms, pl->m2l_tile,
+    e = launch_m2l_tc(pl->hspecM, bp->Gr, pl->hspecL, pl->m2l_tab_tc, pl->p, (int)Kc, Khh, pl->num_sms, pl->m2l_tile,
                       pl->err, s, nl);
   else
     e = launch_m2l_batched(fp64, pl->hspecM, bp->G, pl->hspecL, pl->m2l_tab, pl->p, (int)Kc, Khh, s, nl);
