@@ -292,8 +292,14 @@ __device__ __forceinline__ void pp_pair2_mixed(const ulonglong2& A, const ulongl
 // while the other buffer's copies are in flight.  A wait that runs out
 // raises the device error flag (PMMM_ERR_TIMEOUT), waits once more (bounded) for
 // the copies it issued and leaves the kernel.
-constexpr int NT_CAP = 128;                    // source pairs per buffer (4 KB), a multiple of 4
-constexpr int NT_BLOCKS_PER_SM = 5;            // resident blocks per SM (up to 102 registers per thread)
+// Source pairs per buffer (a multiple of 4) and resident blocks per SM, within 227 KB of
+// shared memory.  The per-chunk work (wait, copies, shifts of the cells that begin or end
+// in it) favours long chunks, the sweeps' latency more blocks.  Near field of 2^20 /
+// 32^3 and 2^24 / 64^3 (c = 1), 2^20 / 32^3 (c = 2): 64 pairs, 6 blocks 557 us, 14.6 ms,
+// 2.81 ms; 96, 6: 541, 14.3, 2.70; 128, 5: 528, 13.9, 2.62; 160, 5: 518, 13.8, 2.58;
+// 192, 4: 549, 14.4, 2.50; 256, 3: 563, 14.3, 2.54.
+template <int CUT> constexpr int nt_cap() { return CUT <= 1 ? 160 : 192; }
+template <int CUT> constexpr int nt_blocks_per_sm() { return CUT <= 1 ? 5 : 4; }
 constexpr long long NT_WAIT_POLLS = 1 << 20;  // polls of at most 1 us each
 
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
@@ -379,13 +385,14 @@ __device__ __forceinline__ void pp_sweep(const float4* __restrict__ src, int npa
 }
 
 template <int CUT>
-__global__ void __launch_bounds__(PP_WARPS * 32, NT_BLOCKS_PER_SM) pp_kernel_tma(
+__global__ void __launch_bounds__(PP_WARPS * 32, nt_blocks_per_sm<CUT>()) pp_kernel_tma(
     const float* __restrict__ part, const float* __restrict__ src2f, const uint32_t* __restrict__ pair_start,
     const uint32_t* __restrict__ vals, const int* __restrict__ cs, int64_t K, const uint32_t* __restrict__ item_start,
     const uint32_t* __restrict__ item_cell, unsigned int* __restrict__ counter, const float* __restrict__ far,
     PPParams pp, float* __restrict__ phi, float* __restrict__ force, double* __restrict__ epart,
     int* __restrict__ err, float4* __restrict__ near_out) {
   constexpr int W = 2 * CUT + 1, NS = W * W * W, SL = (NS + 31) / 32, SELFK = (NS - 1) / 2;
+  constexpr int NT_CAP = nt_cap<CUT>();
   __shared__ __align__(128) float4 sbuf[PP_WARPS][2][2 * NT_CAP];
   __shared__ __align__(8) unsigned long long sbar[PP_WARPS][2];
   const float4* P = reinterpret_cast<const float4*>(part);
@@ -953,9 +960,9 @@ cudaError_t launch_pp(bool fp64, const void* part, const void* src2, const uint3
     if (pp.c <= 1) PP_TARGETS(1); else PP_TARGETS(2);
 #undef PP_TARGETS
   } else {
-    // persistent launch: NT_BLOCKS_PER_SM resident blocks of PP_WARPS warps per SM
+    // persistent launch: nt_blocks_per_sm resident blocks of PP_WARPS warps per SM
 #define PP_ITEMS(C)                                                                                                  \
-  pp_kernel_tma<C><<<(unsigned)(NT_BLOCKS_PER_SM * sms), PP_WARPS * 32, 0, s>>>(                                     \
+  pp_kernel_tma<C><<<(unsigned)(nt_blocks_per_sm<C>() * sms), PP_WARPS * 32, 0, s>>>(                                \
       (const float*)part, (const float*)src2, pair_start, vals, cell_start, K, item_start, item_cell, counter,       \
       (const float*)far, pp, (float*)phi, (float*)force, epart, err, (float4*)near_out)
     if (pp.c <= 1) PP_ITEMS(1); else PP_ITEMS(2);
