@@ -261,10 +261,11 @@ enum {
   PMMM_INFO_M2L_ARITH = 12, /* arithmetic of the last compute's M2L: PMMM_M2L_ARITH_* (-1 before any) */
   PMMM_INFO_SPLIT = 13      /* 1 if the last compute ran the far field beside the near field (below) */
 };
-/* Split evaluation (near_field = PMMM_NEAR_CELL_ITEMS_SPLIT, set in the config or
- * chosen by pmmm_plan_autotune; FP32 plans): after the sort, the far field (P2M,
+/* Split evaluation (FP32 plans; near_field = PMMM_NEAR_CELL_ITEMS_SPLIT, set in the
+ * config or chosen by pmmm_plan_autotune, and PMMM_NEAR_AUTO for small systems, with
+ * whichever near-field kernel it takes): after the sort, the far field (P2M,
  * mesh stage, periodic corrections, L2P) runs on a second stream of the plan,
- * created with the highest priority, beside the cell-item near field, whose sums
+ * created with the highest priority, beside the near field, whose sums
  * go to a workspace buffer (16 bytes per particle, allocated on the first plain
  * call that needs it); one more launch adds the two.  The results equal those of
  * the one-stream sequence bit for bit.  One stream while stage timing is on, for

@@ -161,10 +161,18 @@ cudaError_t alloc_mesh(pmmm_plan* pl, int B) {
 int ensure_particles(pmmm_plan* pl, int64_t n);
 int ensure_m2l_tables(pmmm_plan* pl);
 void set_streams(pmmm_plan* pl, cudaStream_t s);
+// The automatic near field splits evaluations of at most this many particles: there the
+// far field is a chain of launches that leave the GPU mostly idle, and the near field fits
+// beside it (graph-launched evaluations, one stream -> split: 8^3 cells p = 5, 9 / 32 per
+// cell 78 -> 62, 100 -> 68 us; 16^3, 5 / 32 per cell 110 -> 99, 154 -> 148 us; 32^3 p = 7,
+// 4 / 9 / 32 per cell 135 -> 134, 212 -> 213, 704 -> 716 us; 64^3 p = 5, 32: 4.83 -> 5.26 ms).
+constexpr int64_t SPLIT_AUTO_MAX = 1 << 17;
 // the near sums' buffer of the split evaluation is kept once a choice asks for it
-bool wants_split(const pmmm_plan* pl) {
-  return !pl->fp64 && (pl->cfg.near_field == PMMM_NEAR_CELL_ITEMS_SPLIT || pl->tuned_near == PMMM_NEAR_CELL_ITEMS_SPLIT ||
-                       pl->nearv != nullptr);
+bool wants_split(const pmmm_plan* pl, int64_t cap) {
+  if (pl->fp64) return false;
+  return (pl->cfg.near_field == PMMM_NEAR_AUTO && cap <= 8 * SPLIT_AUTO_MAX) ||
+         pl->cfg.near_field == PMMM_NEAR_CELL_ITEMS_SPLIT || pl->tuned_near == PMMM_NEAR_CELL_ITEMS_SPLIT ||
+         pl->nearv != nullptr;
 }
 
 // Grows the mesh workspace to B systems (the particle workspace, sized by the
@@ -245,7 +253,7 @@ int ensure_particles(pmmm_plan* pl, int64_t n) {
   if (e == cudaSuccess) e = dalloc(pl, &v, sizeof(double) * 4 * (size_t)mi);
   if (e == cudaSuccess) pl->epart = (double*)v;
   if (e == cudaSuccess && !pl->fp64) e = dalloc(pl, &pl->src2, 32 * (size_t)pp_pairs_max(Kb, cap));
-  if (e == cudaSuccess && wants_split(pl)) e = dalloc(pl, &pl->nearv, 16 * (size_t)cap);
+  if (e == cudaSuccess && wants_split(pl, cap)) e = dalloc(pl, &pl->nearv, 16 * (size_t)cap);
   // items of one system: at most its cells + cap / 32 + 1
   const int bch = reduce_batched_chunks(pl->d.K, pp_items_max(pl->d.K, cap));
   if (e == cudaSuccess) e = dalloc(pl, &v, sizeof(double) * 5 * (size_t)pl->bcap * bch);
@@ -506,8 +514,8 @@ int run(pmmm_plan* pl, int B, int64_t n, const void* pos, const void* q, void* p
   // and runs beside the near field, which then leaves its sums in nearv; a
   // combination launch follows both.  Not with stage timing (stages queued one
   // by one) nor with a far-field hook (the surrogate's own plans).
-  split = near == PMMM_NEAR_CELL_ITEMS_SPLIT && pl->aux && !pl->timing && !pl->hook && pl->src2 &&
-          pp_tma_applies(fp64, pl->g.c, per_target);
+  split = ((near == PMMM_NEAR_CELL_ITEMS_SPLIT && !per_target) || (near == PMMM_NEAR_AUTO && n <= SPLIT_AUTO_MAX)) &&
+          pl->aux && !pl->timing && !pl->hook && pl->src2;
   if (split && !pl->nearv) {
     // the near sums' buffer, allocated outside a capture (the plan's or the
     // caller's; inside one the evaluation keeps one stream)
@@ -605,8 +613,8 @@ int run(pmmm_plan* pl, int B, int64_t n, const void* pos, const void* q, void* p
                  split ? pl->nearv : nullptr, s, &nl));
     if (split) {
       CK(cudaStreamWaitEvent(s, pl->ev_join, 0));
-      CK(launch_pp_combine(pl->part, pl->vals_sorted, pl->cs, K, pl->item_start, pl->item_cell, mi, pl->far,
-                           pl->nearv, pp, phi, force, pl->epart, pl->num_sms, s, &nl));
+      CK(launch_pp_combine(per_target, pl->part, pl->keys_sorted, pl->vals_sorted, n, pl->cs, K, pl->item_start,
+                           pl->item_cell, mi, pl->far, pl->nearv, pp, phi, force, pl->epart, s, &nl));
     }
     mark(pl, ST_REDUCE);
     if (B == 1)

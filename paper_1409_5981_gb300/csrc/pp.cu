@@ -678,6 +678,77 @@ __global__ void __launch_bounds__(256) pp_combine_kernel(const float4* __restric
   }
 }
 
+constexpr int PPS_THREADS = 256;
+
+// The end of a per-target evaluation for sorted target i (cell, near sums nr): adds the
+// far field, stores the results in the caller's order and reduces the energy and
+// net-force terms per work item -- a segmented warp scan over lanes of equal item, one
+// store per item that lies inside the warp, and two double atomics (commutative, so
+// deterministic) on a zeroed slot for an item split between two warps.  Called by whole
+// warps (i >= n: no target).
+__device__ __forceinline__ void target_epilogue(int64_t i, int64_t n, int cell, float4 nr,
+                                                const float4* __restrict__ P, const uint32_t* __restrict__ vals,
+                                                const int* __restrict__ cs, const uint32_t* __restrict__ item_start,
+                                                const float4* __restrict__ far, const PPParams& pp,
+                                                float* __restrict__ phi, float* __restrict__ force,
+                                                double* __restrict__ epart) {
+  const int lane = threadIdx.x & 31;
+  const int64_t wbase = i - lane;
+  float e_t = 0.f, f_t0 = 0.f, f_t1 = 0.f, f_t2 = 0.f;
+  uint32_t item = 0xffffffffu;
+  int64_t tb = 0, te = 0;
+  if (i < n) {
+    const int c0 = cs[cell], c1 = cs[cell + 1];
+    const int chunk = (int)((i - c0) / CHUNK);
+    item = item_start[cell] + (uint32_t)chunk;
+    tb = c0 + (int64_t)chunk * CHUNK;
+    te = min(tb + CHUNK, (int64_t)c1);
+    const float4 fr = far[i];
+    const float sg = pp.sign32, q = P[i].w;
+    const float pt = sg * (fr.x + nr.x);
+    const float g0 = sg * (fr.y + nr.y), g1 = sg * (fr.z + nr.z), g2 = sg * (fr.w + nr.w);
+    const uint32_t o = vals[i];
+    if (phi) phi[o] = pt;
+    if (force) {
+      force[3 * (int64_t)o + 0] = -q * g0;
+      force[3 * (int64_t)o + 1] = -q * g1;
+      force[3 * (int64_t)o + 2] = -q * g2;
+    }
+    e_t = 0.5f * q * pt;
+    f_t0 = -q * g0;
+    f_t1 = -q * g1;
+    f_t2 = -q * g2;
+  }
+  // segmented inclusive scan over runs of lanes with the same item
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const float ue = __shfl_up_sync(0xffffffffu, e_t, o), u0 = __shfl_up_sync(0xffffffffu, f_t0, o);
+    const float u1 = __shfl_up_sync(0xffffffffu, f_t1, o), u2 = __shfl_up_sync(0xffffffffu, f_t2, o);
+    const uint32_t uit = __shfl_up_sync(0xffffffffu, item, o);
+    if (lane >= o && uit == item) {
+      e_t += ue;
+      f_t0 += u0;
+      f_t1 += u1;
+      f_t2 += u2;
+    }
+  }
+  const uint32_t next = __shfl_down_sync(0xffffffffu, item, 1);
+  if (i < n && (lane == 31 || next != item)) {
+    double* ep = epart + 4 * (int64_t)item;
+    if (tb >= wbase && te <= wbase + 32) {
+      ep[0] = (double)e_t;
+      ep[1] = (double)f_t0;
+      ep[2] = (double)f_t1;
+      ep[3] = (double)f_t2;
+    } else {
+      atomicAdd(ep + 0, (double)e_t);
+      atomicAdd(ep + 1, (double)f_t0);
+      atomicAdd(ep + 2, (double)f_t1);
+      atomicAdd(ep + 3, (double)f_t2);
+    }
+  }
+}
+
 // FP32 near field (c = 1 or 2) with one thread per target: for sparsely filled cells,
 // where the per-item set-up of the cell-item kernels costs more than the
 // interactions.  Thread i takes sorted target i; it walks the (2c+1)^2 neighbour rows
@@ -693,12 +764,8 @@ __global__ void __launch_bounds__(256) pp_combine_kernel(const float4* __restric
 // the pair step's operand reads (33 cycles per 64 pairs and SM quarter) where they are
 // full.  Against one loop per cell and L1 loads throughout: 20011 particles / 16^3 29 ->
 // 20 us; 10^6 / 64^3 195 -> 160 us; 5.6 million in 64 systems 1336 -> 1124 us; 2^20 in a
-// Plummer sphere / 64^3 (3.5e10 pairs, up to 6300 particles per cell) 27.9 -> 18.4 ms.  Energy
-// and net-force terms are reduced per work item: a segmented warp scan over
-// lanes of equal item, one store per item that lies inside the warp, and two
-// double atomics (commutative, so deterministic) on a zeroed slot for an item
-// split between two warps.
-constexpr int PPS_THREADS = 256;
+// Plummer sphere / 64^3 (3.5e10 pairs, up to 6300 particles per cell) 27.9 -> 18.4 ms.
+// near_out (split evaluation): the near sums go there, pp_combine_target_kernel ends.
 
 // Sums of one target over npair pairs whose words lie in sa and sb (shared memory).
 template <bool SELF>
@@ -762,14 +829,10 @@ __global__ void __launch_bounds__(PPS_THREADS, 4) pp_target_kernel(
     const float4* __restrict__ P, const ulonglong2* __restrict__ S2, const uint32_t* __restrict__ pair_start,
     const uint32_t* __restrict__ keys, const uint32_t* __restrict__ vals, const int* __restrict__ cs,
     const uint32_t* __restrict__ item_start, int64_t n, const float4* __restrict__ far, PPParams pp,
-    float* __restrict__ phi, float* __restrict__ force, double* __restrict__ epart) {
+    float* __restrict__ phi, float* __restrict__ force, double* __restrict__ epart, float4* __restrict__ near_out) {
   constexpr int W = 2 * CUT + 1;
   const int64_t i = (int64_t)blockIdx.x * PPS_THREADS + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  const int64_t wbase = i - lane;
-  float e_t = 0.f, f_t0 = 0.f, f_t1 = 0.f, f_t2 = 0.f;
-  uint32_t item = 0xffffffffu;
-  int64_t tb = 0, te = 0;
+  float4 nr = make_float4(0.f, 0.f, 0.f, 0.f);
   __shared__ float4 stage[PPS_THREADS / 32][2][32];
   const int mycell = i < n ? (int)keys[i] : -1;
   const int cell0 = __shfl_sync(0xffffffffu, mycell, 0);  // every lane takes part
@@ -777,11 +840,6 @@ __global__ void __launch_bounds__(PPS_THREADS, 4) pp_target_kernel(
   if (i < n) {
     const float4 xi = P[i];
     const int cell = mycell;
-    const int c0 = cs[cell], c1 = cs[cell + 1];
-    const int chunk = (int)((i - c0) / CHUNK);
-    item = item_start[cell] + (uint32_t)chunk;
-    tb = c0 + (int64_t)chunk * CHUNK;
-    te = min(tb + CHUNK, (int64_t)c1);
     const int nx = pp.n[0], ny = pp.n[1], nz = pp.n[2];
     const int sbase = cell - cell % pp.ksys, lc = cell - sbase;
     const int ix = lc % nx, iy = (lc / nx) % ny, iz = lc / (nx * ny);
@@ -865,51 +923,27 @@ __global__ void __launch_bounds__(PPS_THREADS, 4) pp_target_kernel(
       up2(gz, za, zb);
     }
     const float ps = pa + pbv, gxs = -(xa + xb), gys = -(ya + yb), gzs = -(za + zb);
-    const float4 fr = far[i];
-    const float ih = pp.ih32, ih2 = pp.ih2_32, sg = pp.sign32;
-    const float pt = sg * (fr.x + ps * ih);
-    const float g0 = sg * (fr.y + gxs * ih2), g1 = sg * (fr.z + gys * ih2), g2 = sg * (fr.w + gzs * ih2);
-    const uint32_t o = vals[i];
-    const float q = xi.w;
-    if (phi) phi[o] = pt;
-    if (force) {
-      force[3 * (int64_t)o + 0] = -q * g0;
-      force[3 * (int64_t)o + 1] = -q * g1;
-      force[3 * (int64_t)o + 2] = -q * g2;
-    }
-    e_t = 0.5f * q * pt;
-    f_t0 = -q * g0;
-    f_t1 = -q * g1;
-    f_t2 = -q * g2;
+    // near sums in units of 1 / hs and 1 / hs^2, rounded on their own (as in pp_kernel_tma)
+    nr = make_float4(__fmul_rn(ps, pp.ih32), __fmul_rn(gxs, pp.ih2_32), __fmul_rn(gys, pp.ih2_32),
+                     __fmul_rn(gzs, pp.ih2_32));
   }
-  // segmented inclusive scan over runs of lanes with the same item
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const float ue = __shfl_up_sync(0xffffffffu, e_t, o), u0 = __shfl_up_sync(0xffffffffu, f_t0, o);
-    const float u1 = __shfl_up_sync(0xffffffffu, f_t1, o), u2 = __shfl_up_sync(0xffffffffu, f_t2, o);
-    const uint32_t uit = __shfl_up_sync(0xffffffffu, item, o);
-    if (lane >= o && uit == item) {
-      e_t += ue;
-      f_t0 += u0;
-      f_t1 += u1;
-      f_t2 += u2;
-    }
+  if (near_out) {  // split evaluation: the near sums only, combined later by pp_combine_target_kernel
+    if (i < n) near_out[i] = nr;
+    return;
   }
-  const uint32_t next = __shfl_down_sync(0xffffffffu, item, 1);
-  if (i < n && (lane == 31 || next != item)) {
-    double* ep = epart + 4 * (int64_t)item;
-    if (tb >= wbase && te <= wbase + 32) {
-      ep[0] = (double)e_t;
-      ep[1] = (double)f_t0;
-      ep[2] = (double)f_t1;
-      ep[3] = (double)f_t2;
-    } else {
-      atomicAdd(ep + 0, (double)e_t);
-      atomicAdd(ep + 1, (double)f_t0);
-      atomicAdd(ep + 2, (double)f_t1);
-      atomicAdd(ep + 3, (double)f_t2);
-    }
-  }
+  target_epilogue(i, n, mycell, nr, P, vals, cs, item_start, far, pp, phi, force, epart);
+}
+
+// Combination of a split evaluation with the per-target near field, one thread per
+// sorted target.
+__global__ void __launch_bounds__(PPS_THREADS) pp_combine_target_kernel(
+    const float4* __restrict__ P, const uint32_t* __restrict__ keys, const uint32_t* __restrict__ vals,
+    const int* __restrict__ cs, const uint32_t* __restrict__ item_start, int64_t n, const float4* __restrict__ far,
+    const float4* __restrict__ nearv, PPParams pp, float* __restrict__ phi, float* __restrict__ force,
+    double* __restrict__ epart) {
+  const int64_t i = (int64_t)blockIdx.x * PPS_THREADS + threadIdx.x;
+  const float4 nr = i < n ? nearv[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+  target_epilogue(i, n, i < n ? (int)keys[i] : -1, nr, P, vals, cs, item_start, far, pp, phi, force, epart);
 }
 
 }  // namespace
@@ -919,14 +953,20 @@ int64_t pp_items_max(int64_t K, int64_t n) { return K + (n + CHUNK - 1) / CHUNK 
 int64_t pp_pairs_max(int64_t K, int64_t n) { return (n + K) / 2 + 1; }
 
 bool pp_per_target_applies(bool fp64, int c) { return !fp64 && c <= 2; }
-bool pp_tma_applies(bool fp64, int c, bool per_target) { return !fp64 && c <= 2 && !per_target; }
 
-cudaError_t launch_pp_combine(const void* part, const uint32_t* vals, const int* cell_start, int64_t K,
-                              const uint32_t* item_start, const uint32_t* item_cell, int64_t max_items,
-                              const void* far, const void* nearv, PPParams pp, void* phi, void* force, double* epart,
-                              int num_sms, cudaStream_t s, int* nl) {
+cudaError_t launch_pp_combine(bool per_target, const void* part, const uint32_t* keys, const uint32_t* vals, int64_t n,
+                              const int* cell_start, int64_t K, const uint32_t* item_start, const uint32_t* item_cell,
+                              int64_t max_items, const void* far, const void* nearv, PPParams pp, void* phi, void* force,
+                              double* epart, cudaStream_t s, int* nl) {
+  if (per_target) {
+    if (n <= 0) return cudaSuccess;
+    pp_combine_target_kernel<<<(unsigned)((n + PPS_THREADS - 1) / PPS_THREADS), PPS_THREADS, 0, s>>>(
+        (const float4*)part, keys, vals, cell_start, item_start, n, (const float4*)far, (const float4*)nearv, pp,
+        (float*)phi, (float*)force, epart);
+    ++*nl;
+    return cudaGetLastError();
+  }
   if (max_items <= 0) return cudaSuccess;
-  (void)num_sms;
   const int64_t blocks = (max_items + 7) / 8;  // 8 warps (items) per block, one item per warp
   pp_combine_kernel<<<(unsigned)blocks, 256, 0, s>>>((const float4*)part, vals, cell_start, K, item_start, item_cell,
                                                      (const float4*)far, (const float4*)nearv, pp, (float*)phi,
@@ -942,7 +982,7 @@ cudaError_t launch_pp(bool fp64, const void* part, const void* src2, const uint3
                       cudaStream_t s, int* nl) {
   const int sms = num_sms > 0 ? num_sms : 1;
   if (fp64) {
-    if (near_out) return cudaErrorInvalidValue;  // only the cell-item FP32 kernel splits
+    if (near_out) return cudaErrorInvalidValue;  // only the FP32 kernels split
 #define PP64(C)                                                                                                    \
   pp64_kernel<C><<<(unsigned)(P64_BLOCKS_PER_SM * sms), P64_THREADS, 0, s>>>((const double*)part, vals, cell_start, K, \
                                                                              item_start, item_cell, counter,       \
@@ -956,7 +996,7 @@ cudaError_t launch_pp(bool fp64, const void* part, const void* src2, const uint3
 #define PP_TARGETS(C)                                                                                              \
   pp_target_kernel<C><<<g, PPS_THREADS, 0, s>>>((const float4*)part, (const ulonglong2*)src2, pair_start, keys, vals, \
                                                 cell_start, item_start, n, (const float4*)far, pp, (float*)phi,    \
-                                                (float*)force, epart)
+                                                (float*)force, epart, (float4*)near_out)
     if (pp.c <= 1) PP_TARGETS(1); else PP_TARGETS(2);
 #undef PP_TARGETS
   } else {
