@@ -252,7 +252,7 @@ __device__ __forceinline__ uint32_t crowded_rank(const uint32_t* __restrict__ or
 // its cell plus the number of smaller indices in the cell, and writes there its
 // original index, cell and record; its half of its source pair (PACK: FP32 pair
 // layout, pp.cu), with the dummy partner that completes an odd cell; and the cell of
-// the work item that starts with it.  Also zeroes the energy partials of the unused
+// the work item that starts with it.  Also (epart not null) zeroes the energy partials of the unused
 // item slots (of all of them when the near-field kernel accumulates into them).
 // order is 16-byte aligned and readable up to the next multiple of four entries.
 template <typename V, bool PACK>
@@ -265,8 +265,10 @@ __global__ void __launch_bounds__(RANK_THREADS) rank_gather_kernel(const uint32_
                                                           double4* __restrict__ epart, int64_t max_items,
                                                           int zero_all) {
   const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  for (int64_t i = (zero_all ? 0 : (int64_t)l.item_start[K]) + s; i < max_items; i += (int64_t)gridDim.x * blockDim.x)
-    epart[i] = make_double4(0.0, 0.0, 0.0, 0.0);
+  if (epart)
+    for (int64_t i = (zero_all ? 0 : (int64_t)l.item_start[K]) + s; i < max_items;
+         i += (int64_t)gridDim.x * blockDim.x)
+      epart[i] = make_double4(0.0, 0.0, 0.0, 0.0);
   if (n == 0) return;
   const bool live = s < n;
   uint32_t me = order[live ? s : n - 1], c = keys[me], j = 0;
@@ -344,7 +346,12 @@ cudaError_t launch_cell_sort(const uint32_t* keys, const uint32_t* arrival, uint
                              int64_t max_items, bool zero_all, cudaStream_t s, int* nl) {
   cell_scan_kernel<<<grid1(K + 1, CS_BLK), CS_THREADS, 0, s>>>(count, K, l);
   place_kernel<<<grid1(n > K ? n : K + 1, 256), 256, 0, s>>>(keys, arrival, n, K, l, order);
-  const unsigned blocks = grid1(n > max_items ? n : max_items, RANK_THREADS);
+  const int64_t work = epart && max_items > n ? max_items : n;
+  if (work <= 0) {
+    *nl += 2;
+    return cudaGetLastError();
+  }
+  const unsigned blocks = grid1(work, RANK_THREADS);
   const int za = zero_all ? 1 : 0;
   if (fp64)
     rank_gather_kernel<double4, false><<<blocks, RANK_THREADS, 0, s>>>(order, keys, l, n, K, (const double4*)rec, vals,

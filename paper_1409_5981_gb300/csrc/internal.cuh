@@ -101,7 +101,7 @@ cudaError_t launch_bin_count(const void* pos, const void* q, bool fp64, int64_t 
 // Stable sort by cell with the lists: vals (original index of each sorted slot),
 // keys_sorted (its cell), part[s] = rec[vals[s]] (position relative to the cell centre
 // in units of hs, and the charge), item_cell (the cell of every work item), src2 (FP32:
-// the pair-interleaved sources, 32 bytes per pair, layout in pp.cu) and zeroed energy
+// the pair-interleaved sources, 32 bytes per pair, layout in pp.cu) and, unless epart is null, zeroed energy
 // partials of the unused item slots (of all of them with zero_all: the per-target near
 // field accumulates into them).  count is left zeroed; order: scratch of n + 4 entries,
 // 16-byte aligned.
@@ -356,6 +356,7 @@ int64_t pp_pairs_max(int64_t K, int64_t n);
 // sorted target go to near_out[s] = (phi, grad) / (hs, hs^2) instead of being
 // combined, and launch_pp_combine adds the far field afterwards.
 bool pp_per_target_applies(bool fp64, int c);
+// epart may be null everywhere: no energy and force partials.
 cudaError_t launch_pp(bool fp64, const void* part, const void* src2, const uint32_t* pair_start, const uint32_t* vals,
                       const uint32_t* keys, int64_t n, bool per_target, const int* cell_start, int64_t K,
                       const uint32_t* item_start, const uint32_t* item_cell, unsigned int* counter, int num_sms,

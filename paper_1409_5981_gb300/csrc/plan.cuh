@@ -68,12 +68,18 @@ struct pmmm_plan {
   // CUDA graph of one evaluation, and what it was captured for: the systems'
   // offsets, the caller's pointers, the workspace generation and the tuning
   // choices.  Captured on a private stream, launched on the plan's stream.
-  cudaGraphExec_t gexec = nullptr;
+  // One without and one with the energy reduction, so that a program that reads
+  // the energy now and then does not capture again.
+  struct Graph {
+    cudaGraphExec_t exec = nullptr;
+    std::vector<int64_t> off;
+    const void* ptr[4] = {nullptr, nullptr, nullptr, nullptr};
+    uint64_t gen = 0;
+    int tune[2] = {0, 0};
+  };
+  Graph graph[2];
   cudaStream_t cstream = nullptr;
-  std::vector<int64_t> gkey_off;
-  const void* gkey_ptr[4] = {nullptr, nullptr, nullptr, nullptr};
-  uint64_t gkey_gen = 0;
-  int gkey_tune[2] = {0, 0};
+  bool want_energy = true;  // of the call being made
   bool capturing = false;
   // the last plain single-system call (pmmm_compute takes the graph from the
   // second identical call on)
@@ -123,7 +129,7 @@ struct pmmm_plan {
 
 namespace pmmm {
 // One evaluation of B systems (pmmm.cu); B > 1 needs the offsets uploaded.
-int plan_run(pmmm_plan* pl, int B, int64_t n, const void* pos, const void* q, void* phi, void* force);
+int plan_run(pmmm_plan* pl, int B, int64_t n, const void* pos, const void* q, void* phi, void* force, bool energy);
 int plan_read_energies(pmmm_plan* pl, int B, double* out);
 int plan_map_cuda(cudaError_t e);
 }  // namespace pmmm

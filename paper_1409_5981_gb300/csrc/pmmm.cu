@@ -109,8 +109,10 @@ void free_all(pmmm_plan* pl) {
   if (pl->block) pmmm_plan_destroy(pl->block);
   pl->coarse = pl->block = nullptr;
   dfree(pl, pl->hpos); dfree(pl, pl->hq); dfree(pl, pl->hphi); dfree(pl, pl->hforce);
-  if (pl->gexec) cudaGraphExecDestroy(pl->gexec);
-  pl->gexec = nullptr;
+  for (auto& g : pl->graph) {
+    if (g.exec) cudaGraphExecDestroy(g.exec);
+    g.exec = nullptr;
+  }
   if (pl->cstream) cudaStreamDestroy(pl->cstream);
   pl->cstream = nullptr;
   if (pl->aux) {
@@ -487,6 +489,8 @@ int run(pmmm_plan* pl, int B, int64_t n, const void* pos, const void* q, void* p
                           (near == PMMM_NEAR_PER_TARGET || (near == PMMM_NEAR_AUTO && sparse));
   bool split = false;
   cudaStream_t fs = s;
+  // energy partials and their reduction only for a call that returns the energy
+  double* const epart = pl->want_energy ? pl->epart : nullptr;
 #define CK(x)                    \
   do {                           \
     e = (x);                     \
@@ -508,7 +512,7 @@ int run(pmmm_plan* pl, int B, int64_t n, const void* pos, const void* q, void* p
                         pl->cell_count, pl->far, pl->err, s, &nl));
     CK(launch_cell_sort(pl->keys, pl->vals_sorted, pl->cell_count, pl->far, fp64, n, K, cl, pl->order,
                         pl->vals_sorted, pl->keys_sorted, pl->part, fp64 ? nullptr : pl->src2, pl->item_cell,
-                        pl->epart, pp_items_max(K, n), per_target, s, &nl));
+                        epart, pp_items_max(K, n), per_target, s, &nl));
   }
   // Split evaluation: the far field (P2M .. L2P) goes to the plan's second stream
   // and runs beside the near field, which then leaves its sums in nearv; a
@@ -609,18 +613,20 @@ int run(pmmm_plan* pl, int B, int64_t n, const void* pos, const void* q, void* p
     pp.sign32 = (float)pp.signf;
     const int64_t mi = pp_items_max(K, n);
     CK(launch_pp(fp64, pl->part, pl->src2, pl->pair_start, pl->vals_sorted, pl->keys_sorted, n, per_target, pl->cs, K,
-                 pl->item_start, pl->item_cell, pl->counter, pl->num_sms, pl->far, pp, phi, force, pl->epart, pl->err,
+                 pl->item_start, pl->item_cell, pl->counter, pl->num_sms, pl->far, pp, phi, force, epart, pl->err,
                  split ? pl->nearv : nullptr, s, &nl));
     if (split) {
       CK(cudaStreamWaitEvent(s, pl->ev_join, 0));
       CK(launch_pp_combine(per_target, pl->part, pl->keys_sorted, pl->vals_sorted, n, pl->cs, K, pl->item_start,
-                           pl->item_cell, mi, pl->far, pl->nearv, pp, phi, force, pl->epart, s, &nl));
+                           pl->item_cell, mi, pl->far, pl->nearv, pp, phi, force, epart, s, &nl));
     }
     mark(pl, ST_REDUCE);
-    if (B == 1)
-      CK(launch_energy(pl->epart, mi, pl->partial + 256 * 5, reduce_tickets(pl) + 1, pl->energy, s, &nl));
+    if (!epart)
+      ;
+    else if (B == 1)
+      CK(launch_energy(epart, mi, pl->partial + 256 * 5, reduce_tickets(pl) + 1, pl->energy, s, &nl));
     else
-      CK(launch_energy_batched(pl->epart, pl->item_start, Ks, B, pl->bchunks, pl->bpartial, pl->energy, s, &nl));
+      CK(launch_energy_batched(epart, pl->item_start, Ks, B, pl->bchunks, pl->bpartial, pl->energy, s, &nl));
   }
   mark(pl, ST_COUNT);
 #undef CK
@@ -727,15 +733,16 @@ int graph_eval(pmmm_plan* pl, int B, int64_t n, const int64_t* off, const void* 
                void* force) {
   const void* ptrs[4] = {pos, q, phi, force};
   const uint64_t gen = plan_gen(pl);
-  const bool same = pl->gexec && pl->gkey_off.size() == (size_t)B + 1 &&
-                    memcmp(pl->gkey_off.data(), off, sizeof(int64_t) * (B + 1)) == 0 &&
-                    memcmp(pl->gkey_ptr, ptrs, sizeof(ptrs)) == 0 && pl->gkey_gen == gen &&
-                    pl->gkey_tune[0] == pl->tuned_near && pl->gkey_tune[1] == pl->m2l_tile;
+  pmmm_plan::Graph& g = pl->graph[pl->want_energy ? 1 : 0];
+  const bool same = g.exec && g.off.size() == (size_t)B + 1 &&
+                    memcmp(g.off.data(), off, sizeof(int64_t) * (B + 1)) == 0 &&
+                    memcmp(g.ptr, ptrs, sizeof(ptrs)) == 0 && g.gen == gen &&
+                    g.tune[0] == pl->tuned_near && g.tune[1] == pl->m2l_tile;
   cudaError_t e = cudaSuccess;
   if (!same) {
-    if (pl->gexec) cudaGraphExecDestroy(pl->gexec);
-    pl->gexec = nullptr;
-    pl->gkey_off.clear();
+    if (g.exec) cudaGraphExecDestroy(g.exec);
+    g.exec = nullptr;
+    g.off.clear();
     if (!pl->cstream) {
       e = cudaStreamCreateWithFlags(&pl->cstream, cudaStreamNonBlocking);
       if (e != cudaSuccess) {
@@ -758,20 +765,20 @@ int graph_eval(pmmm_plan* pl, int B, int64_t n, const int64_t* off, const void* 
     set_streams(pl, user);
     // node priorities as captured (the far-field stream's launches first)
     if (e == cudaSuccess && rc == PMMM_OK)
-      e = cudaGraphInstantiateWithFlags(&pl->gexec, graph, cudaGraphInstantiateFlagUseNodePriority);
+      e = cudaGraphInstantiateWithFlags(&g.exec, graph, cudaGraphInstantiateFlagUseNodePriority);
     if (graph) cudaGraphDestroy(graph);
     if (rc != PMMM_OK || e != cudaSuccess) {
-      if (pl->gexec && e != cudaSuccess) cudaGraphExecDestroy(pl->gexec);
-      pl->gexec = nullptr;
+      if (g.exec && e != cudaSuccess) cudaGraphExecDestroy(g.exec);
+      g.exec = nullptr;
       return rc != PMMM_OK ? rc : map_cuda(e);
     }
-    pl->gkey_off.assign(off, off + B + 1);
-    memcpy(pl->gkey_ptr, ptrs, sizeof(ptrs));
-    pl->gkey_gen = gen;
-    pl->gkey_tune[0] = pl->tuned_near;
-    pl->gkey_tune[1] = pl->m2l_tile;
+    g.off.assign(off, off + B + 1);
+    memcpy(g.ptr, ptrs, sizeof(ptrs));
+    g.gen = gen;
+    g.tune[0] = pl->tuned_near;
+    g.tune[1] = pl->m2l_tile;
   }
-  e = cudaGraphLaunch(pl->gexec, pl->stream);
+  e = cudaGraphLaunch(g.exec, pl->stream);
   if (e != cudaSuccess) return map_cuda(e);
   pl->n_last = n;
   pl->nsys_last = B;
@@ -840,7 +847,8 @@ int run_host(pmmm_plan* pl, int B, int64_t n, const void* pos, const void* q, vo
 }  // namespace
 
 namespace pmmm {
-int plan_run(pmmm_plan* pl, int B, int64_t n, const void* pos, const void* q, void* phi, void* force) {
+int plan_run(pmmm_plan* pl, int B, int64_t n, const void* pos, const void* q, void* phi, void* force, bool energy) {
+  pl->want_energy = energy;
   return run(pl, B, n, pos, q, phi, force);
 }
 int plan_read_energies(pmmm_plan* pl, int B, double* out) { return read_energies(pl, B, out); }
@@ -993,6 +1001,7 @@ int pmmm_plan_reserve_batched(pmmm_plan* pl, int32_t nsys, int64_t n) {
 int pmmm_compute(pmmm_plan* pl, int64_t n, const void* pos, const void* q, void* phi, void* force, double* energy) {
   if (!pl || n < 0 || n > INT32_MAX) return PMMM_ERR_INVALID_ARG;
   if (n > 0 && (!pos || !q)) return PMMM_ERR_INVALID_ARG;
+  pl->want_energy = energy != nullptr;
   int rc = run_single(pl, n, pos, q, phi, force);
   if (rc != PMMM_OK) return rc;
   return energy ? read_energies(pl, 1, energy) : PMMM_OK;
@@ -1002,12 +1011,10 @@ int pmmm_compute_host(pmmm_plan* pl, int64_t n, const void* pos, const void* q, 
                       double* energy) {
   if (!pl || n < 0 || n > INT32_MAX) return PMMM_ERR_INVALID_ARG;
   if (n > 0 && (!pos || !q)) return PMMM_ERR_INVALID_ARG;
+  pl->want_energy = energy != nullptr;
   int rc = run_host(pl, 1, n, pos, q, phi, force);
   if (rc != PMMM_OK) return rc;
-  double e = 0.0;
-  rc = read_energies(pl, 1, &e);
-  if (energy) *energy = e;
-  return rc;
+  return energy ? read_energies(pl, 1, energy) : read_device_status(pl);
 }
 
 int pmmm_compute_batched(pmmm_plan* pl, int32_t nsys, const int64_t* offsets, const void* pos, const void* q,
@@ -1018,6 +1025,7 @@ int pmmm_compute_batched(pmmm_plan* pl, int32_t nsys, const int64_t* offsets, co
   int rc = upload_offsets(pl, nsys, offsets, &n);
   if (rc != PMMM_OK) return rc;
   if (n > 0 && (!pos || !q)) return PMMM_ERR_INVALID_ARG;
+  pl->want_energy = energies != nullptr;
   rc = run(pl, nsys, n, pos, q, phi, force);
   if (rc != PMMM_OK) return rc;
   return energies ? read_energies(pl, nsys, energies) : PMMM_OK;
@@ -1031,12 +1039,10 @@ int pmmm_compute_batched_host(pmmm_plan* pl, int32_t nsys, const int64_t* offset
   int rc = upload_offsets(pl, nsys, offsets, &n);
   if (rc != PMMM_OK) return rc;
   if (n > 0 && (!pos || !q)) return PMMM_ERR_INVALID_ARG;
+  pl->want_energy = energies != nullptr;
   rc = run_host(pl, nsys, n, pos, q, phi, force);
   if (rc != PMMM_OK) return rc;
-  std::vector<double> e((size_t)nsys);
-  rc = read_energies(pl, nsys, e.data());
-  if (energies) memcpy(energies, e.data(), sizeof(double) * nsys);
-  return rc;
+  return energies ? read_energies(pl, nsys, energies) : read_device_status(pl);
 }
 
 int pmmm_compute_batched_graph(pmmm_plan* pl, int32_t nsys, const int64_t* offsets, const void* pos, const void* q,
@@ -1049,6 +1055,7 @@ int pmmm_compute_batched_graph(pmmm_plan* pl, int32_t nsys, const int64_t* offse
   if (n > 0 && (!pos || !q)) return PMMM_ERR_INVALID_ARG;
   rc = ensure_particles(pl, n);
   if (rc != PMMM_OK) return rc;
+  pl->want_energy = energies != nullptr;
   rc = graph_eval(pl, nsys, n, offsets, pos, q, phi, force);
   if (rc != PMMM_OK) return rc;
   return energies ? read_energies(pl, nsys, energies) : PMMM_OK;
@@ -1082,6 +1089,7 @@ int pmmm_plan_autotune(pmmm_plan* pl, int32_t nsys, const int64_t* offsets, cons
   }
   const bool timing = pl->timing;
   pl->timing = false;
+  pl->want_energy = false;
   float best = 1e30f;
   int best_near = pl->tuned_near, best_tile = pl->m2l_tile;
   for (int nr : nears)

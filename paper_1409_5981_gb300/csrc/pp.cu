@@ -19,7 +19,6 @@ namespace pmmm {
 namespace {
 
 constexpr int PP_WARPS = 4;
-constexpr int PP_BATCH = 1;  // work items taken per atomic by the FP32 near-field warps (one: the shortest tail)
 constexpr int CHUNK = PP_CHUNK;
 
 // FP32 reciprocal square root: the hardware approximation (PTX rsqrt.approx,
@@ -199,12 +198,12 @@ __global__ void __launch_bounds__(P64_THREADS, P64_BLOCKS_PER_SM) pp64_kernel(
       }
       // deterministic sums of this item's energy and net-force partials
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
+      for (int o = 16; epart && o > 0; o >>= 1) {
         e_t += __shfl_xor_sync(0xffffffffu, e_t, o);
 #pragma unroll
         for (int a = 0; a < 3; ++a) f_t[a] += __shfl_xor_sync(0xffffffffu, f_t[a], o);
       }
-      if (lane == 0) {
+      if (epart && lane == 0) {
         epart[(int64_t)item * 4 + 0] = e_t;
 #pragma unroll
         for (int a = 0; a < 3; ++a) epart[(int64_t)item * 4 + 1 + a] = f_t[a];
@@ -410,13 +409,10 @@ __global__ void __launch_bounds__(PP_WARPS * 32, nt_blocks_per_sm<CUT>()) pp_ker
   const uint32_t nitems = item_start[K];
   const int nx = pp.n[0], ny = pp.n[1], nz = pp.n[2];
   const float csx = pp.cs32[0], csy = pp.cs32[1], csz = pp.cs32[2];
-  uint32_t item = 0, batch_end = 0;
   for (;;) {
-    if (item >= batch_end) {
-      if (lane == 0) item = atomicAdd(counter, (unsigned)PP_BATCH);
-      item = __shfl_sync(0xffffffffu, item, 0);
-      batch_end = item + PP_BATCH;
-    }
+    uint32_t item = 0;
+    if (lane == 0) item = atomicAdd(counter, 1u);  // one item per atomic: the shortest tail
+    item = __shfl_sync(0xffffffffu, item, 0);
     if (item >= nitems) break;  // warp-uniform
     const int cell = (int)item_cell[item];
     const int chunk = (int)(item - item_start[cell]);
@@ -582,7 +578,6 @@ __global__ void __launch_bounds__(PP_WARPS * 32, nt_blocks_per_sm<CUT>()) pp_ker
                 np3 = __fmul_rn(gzs, pp.ih2_32);
     if (near_out) {  // split evaluation: the near sums only, combined later by pp_combine_kernel
       if (active && ph == 0) near_out[tbeg + tl] = make_float4(np0, np1, np2, np3);
-      ++item;
       continue;
     }
     float e_t = 0.f, f_t[3] = {0.f, 0.f, 0.f};
@@ -605,6 +600,7 @@ __global__ void __launch_bounds__(PP_WARPS * 32, nt_blocks_per_sm<CUT>()) pp_ker
       f_t[1] = -q * g1;
       f_t[2] = -q * g2;
     }
+    if (!epart) continue;  // no energy asked for
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       e_t += __shfl_xor_sync(0xffffffffu, e_t, o);
@@ -618,7 +614,6 @@ __global__ void __launch_bounds__(PP_WARPS * 32, nt_blocks_per_sm<CUT>()) pp_ker
       epart[(int64_t)item * 4 + 2] = (double)f_t[1];
       epart[(int64_t)item * 4 + 3] = (double)f_t[2];
     }
-    ++item;
   }
 }
 
@@ -662,6 +657,7 @@ __global__ void __launch_bounds__(256) pp_combine_kernel(const float4* __restric
       f_t[1] = -q * g1;
       f_t[2] = -q * g2;
     }
+    if (!epart) continue;  // no energy asked for
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       e_t += __shfl_xor_sync(0xffffffffu, e_t, o);
@@ -719,6 +715,7 @@ __device__ __forceinline__ void target_epilogue(int64_t i, int64_t n, int cell, 
     f_t1 = -q * g1;
     f_t2 = -q * g2;
   }
+  if (!epart) return;  // no energy asked for
   // segmented inclusive scan over runs of lanes with the same item
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {

@@ -379,8 +379,8 @@ int pmmm_surrogate_set_fallback(pmmm_surrogate* s, int on) {
 int pmmm_surrogate_training_pair(pmmm_surrogate* s, int64_t n, const void* pos, const void* q, void* X, float* T,
                                  double* stats) {
   if (!s || !X || !T || n < 0 || n > INT32_MAX || (n > 0 && (!pos || !q))) return PMMM_ERR_INVALID_ARG;
-  int rc = plan_run(s->lo, 1, n, pos, q, nullptr, nullptr);
-  if (rc == PMMM_OK) rc = plan_run(s->hi, 1, n, pos, q, nullptr, nullptr);
+  int rc = plan_run(s->lo, 1, n, pos, q, nullptr, nullptr, false);
+  if (rc == PMMM_OK) rc = plan_run(s->hi, 1, n, pos, q, nullptr, nullptr, false);
   if (rc != PMMM_OK) return rc;
   int nl = 0;
   cudaStream_t st = s->stream;
@@ -469,7 +469,7 @@ int pmmm_surrogate_compute(pmmm_surrogate* s, int64_t n, const void* pos, const 
   s->hook.p_l2p = s->p_hi;
   s->hook.L = s->Lcorr;
   s->lo->hook = &s->hook;
-  rc = plan_run(s->lo, 1, n, pos, q, phi, force);
+  rc = plan_run(s->lo, 1, n, pos, q, phi, force, energy != nullptr);
   s->lo->hook = nullptr;
   if (rc != PMMM_OK) return rc;
   if (!energy) return PMMM_OK;
