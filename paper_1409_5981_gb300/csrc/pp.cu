@@ -394,6 +394,7 @@ __global__ void __launch_bounds__(PP_WARPS * 32, nt_blocks_per_sm<CUT>()) pp_ker
   constexpr int NT_CAP = nt_cap<CUT>();
   __shared__ __align__(128) float4 sbuf[PP_WARPS][2][2 * NT_CAP];
   __shared__ __align__(8) unsigned long long sbar[PP_WARPS][2];
+  __shared__ uint32_t soff[PP_WARPS][NS];  // cell offset of the r-th non-empty segment, a signed byte per axis
   const float4* P = reinterpret_cast<const float4*>(part);
   const char* S2 = reinterpret_cast<const char*>(src2f);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -432,13 +433,12 @@ __global__ void __launch_bounds__(PP_WARPS * 32, nt_blocks_per_sm<CUT>()) pp_ker
     // (global), pair count, first pair in the item's numbering, and the shift that
     // moves the cell's sources into the target cell's frame.  The numbering pads the
     // own cell and the whole list to multiples of 4 pairs with zero-charge dummies.
-    int gb[SL], gn[SL], gf[SL];
-    float gsx[SL], gsy[SL], gsz[SL];
+    int gb[SL], gn[SL], gf[SL], nfull = 0;
 #pragma unroll
     for (int j = 0; j < SL; ++j) {
       const int sg = lane + 32 * j;
       gb[j] = gn[j] = 0;
-      gsx[j] = gsy[j] = gsz[j] = 0.f;
+      uint32_t ofs = 0;
       if (sg < NS) {
         const int kk = sg == 0 ? SELFK : (sg - 1 >= SELFK ? sg : sg - 1);
         const int dx = kk % W - CUT, dy = (kk / W) % W - CUT, dz = kk / (W * W) - CUT;
@@ -452,10 +452,11 @@ __global__ void __launch_bounds__(PP_WARPS * 32, nt_blocks_per_sm<CUT>()) pp_ker
           gb[j] = (int)__ldg(pair_start + cj);
           gn[j] = (int)__ldg(pair_start + cj + 1) - gb[j];
         }
-        gsx[j] = (float)dx * csx;
-        gsy[j] = (float)dy * csy;
-        gsz[j] = (float)dz * csz;
+        ofs = (uint32_t)(dx & 255) | ((uint32_t)(dy & 255) << 8) | ((uint32_t)(dz & 255) << 16);
       }
+      const uint32_t full = __ballot_sync(0xffffffffu, gn[j] > 0);
+      if (gn[j] > 0) soff[warp][nfull + __popc(full & ((1u << lane) - 1u))] = ofs;
+      nfull += __popc(full);
     }
     const int nself = __shfl_sync(0xffffffffu, gn[0], 0);
     const int nselfp = (nself + 3) & ~3;  // own cell, padded: [0, nselfp)
@@ -494,7 +495,7 @@ __global__ void __launch_bounds__(PP_WARPS * 32, nt_blocks_per_sm<CUT>()) pp_ker
     for (int c0 = 0; c0 < 2 && c0 < nch; ++c0) issue(c0, c0);
     float2 pot = make_float2(0.f, 0.f), gx = pot, gy = pot, gz = pot;
     const float2 tx = make_float2(xi.x, xi.x), ty = make_float2(xi.y, xi.y), tz = make_float2(xi.z, xi.z);
-    int sc = 1;  // first segment not yet moved into the target's frame
+    int nbeg = 0;  // non-empty segments that begin before the current group of 32 pairs
     bool ok = true;
     for (int ch = 0; ch < nch; ++ch) {
       const int b = ch & 1;
@@ -520,28 +521,22 @@ __global__ void __launch_bounds__(PP_WARPS * 32, nt_blocks_per_sm<CUT>()) pp_ker
         buf[2 * (e - base)] = far4;
         buf[2 * (e - base) + 1] = farq;
       }
-      // the neighbour cells' sources of this chunk moved into the target cell's frame
-      while (sc < NS) {
-        const int j = sc >> 5, src = sc & 31;
-        int f = gf[0], n = gn[0];
-        float sx = gsx[0], sy = gsy[0], sz = gsz[0];
+      // the neighbour cells' sources of this chunk moved into the target cell's frame, 32
+      // pairs at a time whatever their cells: the segment of a pair is the number of
+      // segments that begin at or before it (one pass per segment, half of its lanes idle
+      // at 16 pairs per cell: 2^20 / 32^3 518 us, c = 2 2.50 ms against 494 us, 2.30 ms)
+      for (int e0 = base; e0 < end; e0 += 32) {
+        uint32_t begins = 0;
 #pragma unroll
-        for (int q = 1; q < SL; ++q)
-          if (j == q) {
-            f = gf[q];
-            n = gn[q];
-            sx = gsx[q];
-            sy = gsy[q];
-            sz = gsz[q];
-          }
-        f = __shfl_sync(0xffffffffu, f, src);
-        if (f >= end) break;  // the segment starts in a later chunk
-        n = __shfl_sync(0xffffffffu, n, src);
-        sx = __shfl_sync(0xffffffffu, sx, src);
-        sy = __shfl_sync(0xffffffffu, sy, src);
-        sz = __shfl_sync(0xffffffffu, sz, src);
-        const int lo = max(f, base), hi = min(f + n, end);
-        for (int e = lo + lane; e < hi; e += 32) {
+        for (int j = 0; j < SL; ++j)
+          if (gn[j] > 0 && (uint32_t)(gf[j] - e0) < 32u) begins |= 1u << (gf[j] - e0);
+        begins = __reduce_or_sync(0xffffffffu, begins);
+        const int e = e0 + lane, r = nbeg + __popc(begins & (0xffffffffu >> (31 - lane))) - 1;
+        nbeg += __popc(begins);
+        if (e >= nselfp && e < min(end, real_end)) {
+          const uint32_t ofs = soff[warp][r];
+          const float sx = (float)(signed char)(ofs & 255u) * csx, sy = (float)(signed char)((ofs >> 8) & 255u) * csy,
+                      sz = (float)(signed char)((ofs >> 16) & 255u) * csz;
           float4 A = buf[2 * (e - base)], B = buf[2 * (e - base) + 1];
           A.x += sx;
           A.y += sx;
@@ -552,8 +547,6 @@ __global__ void __launch_bounds__(PP_WARPS * 32, nt_blocks_per_sm<CUT>()) pp_ker
           buf[2 * (e - base)] = A;
           buf[2 * (e - base) + 1] = B;
         }
-        if (f + n > end) break;  // the segment continues in the next chunk
-        ++sc;
       }
       __syncwarp();
       // own-cell pairs (self pair masked), then the rest of the chunk in one sweep
