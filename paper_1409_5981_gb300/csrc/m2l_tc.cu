@@ -30,7 +30,10 @@
 // at C = 64) and by the assembly of W for few.
 // A two-level evaluation of 2^20 particles (2304 wavevectors x 512 systems) 2.20 -> 1.99 ms,
 // 64 systems of 32^3 cells 4.08 -> 3.93 ms against the complex form of one 512-thread CTA
-// per SM that assembled a 128 x 128 W for every tile.
+// per SM that assembled a 128 x 128 W for every tile.  The rest was instruction issue (1694
+// warp instructions a tile, 56 % of the issue slots at 37 % of the memory's): addresses as
+// 32-bit offsets within a wavevector's block and the odd orders as one constant bit mask,
+// 1.98 -> 1.91 ms and 3.87 -> 3.84 ms.
 // Shared-memory operands use the no-swizzle K-major layout of core matrices
 // (8 rows x 16 bytes): element (r, k) at (r/8)*SBO + (k/8)*LBO + (r%8)*16 + (k%8)*2
 // with LBO = 128 B and SBO = 1024 B.  Every mbarrier wait is bounded; on a
@@ -90,9 +93,9 @@ __device__ __forceinline__ void cp4(uint32_t saddr, const void* g) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(saddr), "l"(g) : "memory");
 }
 
-__device__ __forceinline__ bool odd_order(int c) {  // channel c = l(l+1)+m: l odd (c < 64)
-  return (c >= 1 && c < 4) || (c >= 9 && c < 16) || (c >= 25 && c < 36) || c >= 49;
-}
+// bit c set: channel c = l(l+1)+m has an odd order l (c in [l^2, (l+1)^2), c < 64)
+constexpr uint64_t TC_ODD = (((1ull << 4) - 1) ^ ((1ull << 1) - 1)) | (((1ull << 16) - 1) ^ ((1ull << 9) - 1)) |
+                            (((1ull << 36) - 1) ^ ((1ull << 25) - 1)) | (~0ull ^ ((1ull << 49) - 1));
 
 // Entry table (build_m2l_table_tc): index 1 | index 2 << 10 | sign 2 << 30 | sign 1 << 31.
 // nt: systems per tile (at most TC_NT).
@@ -136,19 +139,24 @@ __global__ void __launch_bounds__(TC_THREADS, TC_CTAS_PER_SM)
   const uint32_t idesc = tc::idesc_bf16_m128(TC_CH);
   const uint32_t sbase = smem_u32(smem);
 
+  // Per element the loops below run a handful of instructions (offsets within a wavevector's
+  // block in 32 bits, the odd orders as bit masks of this thread's channels); index
+  // arithmetic in 64 bits and range tests per channel had been two thirds of the kernel's
+  // 1700 instructions per thread and tile.
+  const uint32_t oddx[2] = {(uint32_t)(TC_ODD >> (8 * (tid >> 6))) & 255u,
+                            (uint32_t)(TC_ODD >> (8 * ((tid + TC_THREADS) >> 6))) & 255u};
   // X of one tile: unit (system n, K-group cg of 8 channels)
   float2 xm[2][8];
   auto load_x = [&](int64_t k, int t) {
+    const float2* Mk = Mt + k * C * B;
+    const int n = tid & 63, nch = n < min(nt, B - t * nt) ? C : 0;
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-      const int u = tid + q * TC_THREADS, n = u & 63, cg = u >> 6;
-      const bool live = n < min(nt, B - t * nt);
+      const int c0 = 8 * ((tid + q * TC_THREADS) >> 6);
+      uint32_t off = (uint32_t)(c0 * B + t * nt + n);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int ci = cg * 8 + j;
-        xm[q][j] = make_float2(0.f, 0.f);
-        if (live && ci < C) xm[q][j] = __ldg(Mt + (k * C + ci) * B + (int64_t)t * nt + n);
-      }
+      for (int j = 0; j < 8; ++j, off += (uint32_t)B)
+        xm[q][j] = c0 + j < nch ? __ldg(Mk + off) : make_float2(0.f, 0.f);
     }
   };
   // drains accumulator `buf` (wavevector k, tile t): warp w reads TMEM lanes 32 (w % 4) ... and
@@ -158,22 +166,24 @@ __global__ void __launch_bounds__(TC_THREADS, TC_CTAS_PER_SM)
     const bool done = tc::bar_wait(smem_u32(&bars[buf]), parity, TC_WAIT_LIMIT);
     if (!__all_sync(0xffffffffu, done)) return false;
     tc::fence_after();
-    const int row = 32 * (warp & 3) + lane, n = row >> 1, part = row & 1;
-    const bool live = n < min(nt, B - t * nt);
+    const int row = 32 * (warp & 3) + lane, n = row >> 1;
+    const uint32_t part = row & 1;
+    const int nch = n < min(nt, B - t * nt) ? C : 0;
+    float* Lk = Lt + 2 * k * C * B;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int c0 = 32 * (warp >> 2) + 16 * h;
+      const uint32_t odd = (uint32_t)(TC_ODD >> c0);
+      uint32_t off = 2u * (uint32_t)(c0 * B + t * nt + n);
       float v[16];
       tc::ld16(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(buf * TC_CH + c0), v);
       tc::wait_ld();
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const int c = c0 + j;
+      for (int j = 0; j < 16; ++j, off += 2u * (uint32_t)B) {
         // odd orders: L = i D, so the real part of D is the imaginary part of L and the
         // imaginary part of D minus the real part of L
-        const bool odd = odd_order(c);
-        const float val = odd && part ? -v[j] : v[j];
-        if (live && c < C) Lt[2 * ((k * C + c) * B + (int64_t)t * nt + n) + (odd ? 1 - part : part)] = val;
+        const uint32_t o = (odd >> j) & 1u;
+        if (c0 + j < nch) Lk[off + (part ^ o)] = __uint_as_float(__float_as_uint(v[j]) ^ ((part & o) << 31));
       }
     }
     tc::fence_before();
@@ -217,7 +227,7 @@ __global__ void __launch_bounds__(TC_THREADS, TC_CTAS_PER_SM)
         float xr[8], xi[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          const bool odd = odd_order(cg * 8 + j);  // times i
+          const bool odd = (oddx[q] >> j) & 1u;  // times i
           xr[j] = odd ? -xm[q][j].y : xm[q][j].x;
           xi[j] = odd ? xm[q][j].x : xm[q][j].y;
         }
