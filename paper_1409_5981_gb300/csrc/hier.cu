@@ -19,6 +19,7 @@
 // Device units: lengths in units of the fine cell size hs_f, M_l in units of
 // hs^-l, L_l in units of hs^(l+1) of its level (hs_c = r hs_f), hence the
 // powers of r in the L2L below.
+#include "fft.cuh"
 #include "harmonics.cuh"
 #include "internal.cuh"
 
@@ -177,35 +178,95 @@ __global__ void __launch_bounds__(256) block_forward_kernel(const T* __restrict_
   }
 }
 
+// cos(2 pi j / 32), j = 0 ... 8, and from it exp(s 2 pi i j / N) for N = 2 ... 32
+// (j and N constants after unrolling).
+__host__ __device__ constexpr double cos32(int j) {
+  j &= 31;
+  if (j > 16) j = 32 - j;
+  const double q[9] = {1.0, 0.98078528040323044913, 0.92387953251128675613, 0.83146961230254523708,
+                       0.70710678118654752440, 0.55557023301960222474, 0.38268343236508977173,
+                       0.19509032201612826785, 0.0};
+  return j <= 8 ? q[j] : -q[16 - j];
+}
+template <typename T, int N, int SGN>
+__device__ __forceinline__ cpx<T> rotate(cpx<T> v, int j) {
+  const int k = (j * (32 / N)) & 31;
+  if (k == 0) return v;
+  if (k == 16) return mk(-v.x, -v.y);
+  if (k == 8) return SGN > 0 ? mk(-v.y, v.x) : mk(v.y, -v.x);
+  if (k == 24) return SGN > 0 ? mk(v.y, -v.x) : mk(-v.y, v.x);
+  const T c = (T)cos32(k), sn = (T)(SGN > 0 ? cos32(k + 24) : -cos32(k + 24));  // sin(t) = cos(t - pi/2)
+  return mk(v.x * c - v.y * sn, v.x * sn + v.y * c);
+}
+
+// DFT of length N = 2 ... 32 in registers, exp(SGN 2 pi i j k / N), natural order on
+// both sides, every twiddle a constant.
+template <typename T, int N, int SGN>
+__device__ __forceinline__ void dft_reg(cpx<T>* v) {
+  if constexpr (N == 2) {
+    dft2(v);
+  } else if constexpr (N == 4) {
+    dft4(v, SGN);
+  } else if constexpr (N == 8) {
+    dft8(v, SGN);
+  } else {
+    constexpr int A = 4, B = N / 4;  // n = B n1 + n2, k = k1 + A k2
+    cpx<T> t[A][B];
+#pragma unroll
+    for (int n2 = 0; n2 < B; ++n2) {
+      cpx<T> a[A];
+#pragma unroll
+      for (int n1 = 0; n1 < A; ++n1) a[n1] = v[B * n1 + n2];
+      dft4(a, SGN);
+#pragma unroll
+      for (int k1 = 0; k1 < A; ++k1) t[k1][n2] = rotate<T, N, SGN>(a[k1], n2 * k1);
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < A; ++k1) {
+      dft_reg<T, B, SGN>(t[k1]);
+#pragma unroll
+      for (int k2 = 0; k2 < B; ++k2) v[k1 + A * k2] = t[k1][k2];
+    }
+  }
+}
+
+constexpr int BLK_THREADS = 288;  // of the transforms with compile-time lengths
+
 constexpr int fwd_ns(int M, int R, int esz) {
   // cells per block of the compile-time forward: the largest power of two <= 16 whose
-  // shared arrays (twiddles, x-pass, y-pass, inputs) stay within 100 KB
+  // shared arrays (twiddles, y-pass, inputs) stay within 100 KB
   int ns = 16;
-  while (ns > 1 && (size_t)(2 * esz) * (M + ns * (M / 2 + 1) * R * R + ns * (M / 2 + 1) * M * R) +
-                           (size_t)esz * ns * R * R * R > 100 * 1024)
+  while (ns > 1 && (size_t)(2 * esz) * (M + ns * (M / 2 + 1) * M * R) + (size_t)esz * ns * R * R * R > 100 * 1024)
     ns /= 2;
   return ns;
 }
 
-// The forward of block_forward_kernel with the transform length M, the
-// refinement R and the cells per block NS known at compile time (all index
-// arithmetic by constants).
+// The forward of block_forward_kernel with the transform length M, the refinement R and
+// the cells per block NS known at compile time.  One thread per column: (kx, e, cell)
+// does the x and y passes (R reals to one x frequency, then R values to M outputs),
+// (ky, kx, cell) the z pass, whose M outputs go straight to global memory.  The M
+// outputs of R inputs are M / R twiddled R-point DFTs: k = (M/R) q + t is the q-th output
+// of the DFT of x_e w_M^(te).
+// Bound by the stores of the spectra (64 channels of 2304 wavevectors x 512 cells, 604 MB,
+// 90 us at the copy rate).  Instead of one thread per output with R products and as many
+// shared-memory reads each: forward stage of 2^20 particles, r = 4, p = 7
+// (coarse P2M and transforms included) 308 -> 189 us.
 template <typename T, int M, int R>
-__global__ void __launch_bounds__(256) block_forward_ct_kernel(const T* __restrict__ Mf, cpx<T>* __restrict__ spec,
-                                                               const cpx<T>* __restrict__ tw_g, BlockGeo g) {
-  constexpr int NS = fwd_ns(M, R, sizeof(T)), HX = M / 2 + 1, R3 = R * R * R, KHH = M * M * HX;
+__global__ void __launch_bounds__(BLK_THREADS) block_forward_ct_kernel(const T* __restrict__ Mf,
+                                                                       cpx<T>* __restrict__ spec,
+                                                                       const cpx<T>* __restrict__ tw_g, BlockGeo g) {
+  constexpr int NS = fwd_ns(M, R, sizeof(T)), HX = M / 2 + 1, R3 = R * R * R, KHH = M * M * HX, Q = M / R;
   extern __shared__ unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
-  cpx<T>* A = tw + M;                          // [HX][R(b)][R(e)][NS]
-  cpx<T>* B = A + NS * HX * R * R;             // [HX][M(ky)][R(e)][NS]
+  cpx<T>* B = tw + M;                                // [M(ky)][HX(kx)][R(e)][NS]
   T* x = reinterpret_cast<T*>(B + NS * HX * M * R);  // [R^3][NS]
   const int ch = blockIdx.y;
   const int64_t S0 = (int64_t)blockIdx.x * NS;
   const int tid = threadIdx.x;
-  for (int i = tid; i < M; i += 256) tw[i] = tw_g[i];
-  for (int i = tid; i < NS * R3; i += 256) {
-    const int a = i / NS, s = i % NS;
-    const int ax = a % R, ay = (a / R) % R, az = a / (R * R);
+  for (int i = tid; i < M; i += BLK_THREADS) tw[i] = tw_g[i];
+  for (int i = tid; i < NS * R3; i += BLK_THREADS) {
+    // consecutive threads take the R fine cells of a row of consecutive coarse cells
+    const int ax = i % R, s = (i / R) % NS, ay = (i / (R * NS)) % R, az = i / (R * NS * R);
     const int64_t S = S0 + s;
     T v = T(0);
     if (S < g.Kc) {
@@ -213,46 +274,56 @@ __global__ void __launch_bounds__(256) block_forward_ct_kernel(const T* __restri
       const int64_t f = (int64_t)(Sx * R + ax) + (int64_t)g.nf[0] * ((Sy * R + ay) + (int64_t)g.nf[1] * (Sz * R + az));
       v = Mf[(int64_t)ch * g.Kf + f];
     }
-    x[i] = v;
+    x[(ax + R * (ay + R * az)) * NS + s] = v;
   }
   __syncthreads();
-  for (int i = tid; i < NS * HX * R * R; i += 256) {
-    const int s = i % NS, be = i / NS, e = be % R, b = (be / R) % R, kx = be / (R * R);
-    cpx<T> acc = mk(T(0), T(0));
+  for (int i = tid; i < NS * HX * R; i += BLK_THREADS) {
+    const int s = i % NS, e = (i / NS) % R, kx = i / (NS * R);
+    const T* xe = x + e * R * R * NS + s;
+    cpx<T> v[R], w[R];
 #pragma unroll
-    for (int a = 0; a < R; ++a) {
-      const T v = x[(a + R * (b + R * e)) * NS + s];
-      const cpx<T> w = tw[(kx * a) & (M - 1)];
-      acc.x += v * w.x;
-      acc.y += v * w.y;
+    for (int a = 1; a < R; ++a) w[a] = tw[(kx * a) & (M - 1)];
+#pragma unroll
+    for (int b = 0; b < R; ++b) {
+      v[b] = mk(xe[b * R * NS], T(0));
+#pragma unroll
+      for (int a = 1; a < R; ++a) {
+        const T xa = xe[(a + R * b) * NS];
+        v[b].x += xa * w[a].x;
+        v[b].y += xa * w[a].y;
+      }
     }
-    A[i] = acc;
-  }
-  __syncthreads();
-  for (int i = tid; i < NS * HX * M * R; i += 256) {
-    const int s = i % NS, q = i / NS, e = q % R, ky = (q / R) % M, kx = q / (R * M);
-    const cpx<T>* Ar = A + (kx * R * R + e) * NS + s;
-    cpx<T> acc = mk(T(0), T(0));
+    cpx<T>* o = B + ((size_t)kx * R + e) * NS + s;
 #pragma unroll
-    for (int b = 0; b < R; ++b) cmac(acc, Ar[b * R * NS], tw[(ky * b) & (M - 1)]);
-    B[i] = acc;
+    for (int t = 0; t < Q; ++t) {
+      cpx<T> u[R];
+#pragma unroll
+      for (int b = 0; b < R; ++b) u[b] = rotate<T, M, -1>(v[b], t * b);
+      dft_reg<T, R, -1>(u);
+#pragma unroll
+      for (int q = 0; q < R; ++q) o[(Q * q + t) * HX * R * NS] = u[q];
+    }
   }
   __syncthreads();
   const int64_t ncell = g.Kc - S0 < NS ? g.Kc - S0 : NS;
-  const int64_t rowstride = g.wavemajor ? (int64_t)g.C * g.Kc : 1;
+  const int64_t kstride = g.wavemajor ? (int64_t)g.C * g.Kc : 1;
   cpx<T>* out = g.wavemajor ? spec + (int64_t)ch * g.Kc + S0 : spec + ((int64_t)ch * g.Kc + S0) * KHH;
-  for (int i = tid; i < KHH * NS; i += 256) {
-    const int s = i % NS, k = i / NS;
+  for (int i = tid; i < NS * HX * M; i += BLK_THREADS) {
+    const int s = i % NS, j = i / NS;  // j = ky HX + kx, wavevector k = kz M HX + j
     if (s >= ncell) continue;
-    const int kx = k % HX, kyz = k / HX, ky = kyz % M, kz = kyz / M;
-    const cpx<T>* Br = B + ((kx * M + ky) * R) * NS + s;
-    cpx<T> acc = mk(T(0), T(0));
+    cpx<T> v[R];
 #pragma unroll
-    for (int e = 0; e < R; ++e) cmac(acc, Br[e * NS], tw[(kz * e) & (M - 1)]);
-    if (g.wavemajor)
-      out[k * rowstride + s] = acc;
-    else
-      out[(int64_t)s * KHH + k] = acc;
+    for (int e = 0; e < R; ++e) v[e] = B[(j * R + e) * NS + s];
+    cpx<T>* o = out + (g.wavemajor ? (int64_t)s : (int64_t)s * KHH) + j * kstride;
+#pragma unroll
+    for (int t = 0; t < Q; ++t) {
+      cpx<T> u[R];
+#pragma unroll
+      for (int e = 0; e < R; ++e) u[e] = rotate<T, M, -1>(v[e], t * e);
+      dft_reg<T, R, -1>(u);
+#pragma unroll
+      for (int q = 0; q < R; ++q) o[(Q * q + t) * (M * HX) * kstride] = u[q];
+    }
   }
 }
 
@@ -383,130 +454,105 @@ __global__ void __launch_bounds__(1024) block_inverse_reg_kernel(const cpx<T>* _
   }
 }
 
-constexpr int bitrev(int v, int bits) {
-  int r = 0;
-  for (int b = 0; b < bits; ++b) r |= ((v >> b) & 1) << (bits - 1 - b);
-  return r;
-}
-constexpr int ilog2(int v) { return v <= 1 ? 0 : 1 + ilog2(v / 2); }
-
-// In-register radix-2 inverse DFT of length M (exp(+2 pi i j k / M), unnormalised):
-// v holds the input in bit-reversed order and returns the output in natural order;
-// wp[j] = exp(+2 pi i j / M).
-template <typename T, int M>
-__device__ __forceinline__ void ifft_reg(cpx<T>* v, const cpx<T>* wp) {
-#pragma unroll
-  for (int len = 2; len <= M; len <<= 1) {
-    const int half = len / 2, step = M / len;
-#pragma unroll
-    for (int i = 0; i < M; i += len)
-#pragma unroll
-      for (int j = 0; j < half; ++j) {
-        const cpx<T> a = v[i + j], b = v[i + j + half] * wp[j * step];
-        v[i + j] = a + b;
-        v[i + j + half] = a - b;
-      }
-  }
-}
-
-// Inverse of the block convolution by FFTs along z and y (M-point, in
-// registers, one thread per column) and a direct Hermitian-weighted real
-// transform along x, for the kept outputs only (W per axis at t = u - CR).  The
-// block's whole half spectrum sits in shared memory as F[kz][ky][kx][cell]
-// (cell fastest, the order of the wavevector-major spectra), the z and y passes
-// overwrite their own columns in place with the W kept values.
-constexpr int inv_ns(int M, int esz) {
-  // cells per block of the FFT inverse: the largest power of two <= 8 whose half
-  // spectra stay within 100 KB (one cell when a single one needs more)
+// Inverse of the block convolution by register DFTs, one thread per column: z (M points
+// straight from global memory, the W kept values to shared memory), y (in place) and x (a
+// real transform of M points through a complex one of M / 2), for the kept outputs only (W
+// per axis at t = u - CR, both even).  Shared memory holds F[uz][ky][kx][cell] (cell
+// fastest, the order of the wavevector-major spectra); the x pass leaves its outputs in
+// place, two per complex slot, and the block copies them out in rows.
+// Bound by the reads of the spectra (604 MB as above) and the instructions of the
+// transforms.  Instead of a staged copy of the whole half spectrum, table twiddles, a direct
+// x transform and 4-byte stores 48 bytes apart, and with LM_CO channels per thread in
+// local_matrix_kernel: inverse stage of 2^20 particles, r = 4, p = 7, 604 -> 404 us.
+constexpr size_t kInvSmem = 112 * 1024;  // two blocks per SM
+constexpr size_t inv_smem(int M, int W, int esz, int ns) { return (size_t)(2 * esz) * ns * W * M * (M / 2 + 1); }
+constexpr int inv_ns(int M, int W, int esz) {
+  // cells per block: the largest power of two <= 8 that fits
   int ns = 8;
-  while (ns > 1 && (size_t)(2 * esz) * (M + ns * M * M * (M / 2 + 1)) > 100 * 1024) ns /= 2;
+  while (ns > 1 && inv_smem(M, W, esz, ns) > kInvSmem) ns /= 2;
   return ns;
 }
 
 template <typename T, int M, int W, int CR>
-__global__ void __launch_bounds__(256) block_inverse_fft_kernel(const cpx<T>* __restrict__ spec,
-                                                                T* __restrict__ region,
-                                                                const cpx<T>* __restrict__ tw_g, BlockGeo g) {
+__global__ void __launch_bounds__(BLK_THREADS, 2) block_inverse_fft_kernel(const cpx<T>* __restrict__ spec,
+                                                                           T* __restrict__ region, BlockGeo g) {
   extern __shared__ unsigned char smem_raw[];
-  constexpr int NS = inv_ns(M, sizeof(T));
-  constexpr int HX = M / 2 + 1, LB = ilog2(M), W3 = W * W * W;
-  cpx<T>* wp = reinterpret_cast<cpx<T>*>(smem_raw);  // exp(+2 pi i j / M)
-  cpx<T>* F = wp + M;                                 // [M(kz)][M(ky)][HX(kx)][NS]
+  constexpr int NS = inv_ns(M, W, sizeof(T));
+  constexpr int HX = M / 2 + 1, W3 = W * W * W, MH = M * HX;
+  static_assert(W % 2 == 0 && CR % 2 == 0 && W / 2 <= HX, "outputs in pairs, in place");
+  cpx<T>* F = reinterpret_cast<cpx<T>*>(smem_raw);  // [W(uz)][M(ky)][HX(kx)][NS]
   const int ch = blockIdx.y;
   const int64_t S0 = (int64_t)blockIdx.x * NS;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  constexpr int NCOL = NS * HX * M;  // columns (ky, kx, cell) of the z pass
-  for (int i = tid; i < M; i += nt) wp[i] = conjg(tw_g[i]);
+  const int tid = threadIdx.x;
+  const int ncell = (int)(g.Kc - S0 < NS ? g.Kc - S0 : NS);
+  // z pass: column (ky, kx, cell) -> kept rows uz < W
   {
-    const int64_t ncell = g.Kc - S0 < NS ? g.Kc - S0 : NS;
-    const int64_t rowstride = g.wavemajor ? (int64_t)g.C * g.Kc : 1;
-    const cpx<T>* in = g.wavemajor ? spec + (int64_t)ch * g.Kc + S0 : spec + ((int64_t)ch * g.Kc + S0) * (M * M * HX);
-    for (int i = tid; i < M * NCOL; i += nt) {
-      const int si = i % NS, k = i / NS;  // k = (kz M + ky) HX + kx
-      F[i] = si < ncell ? (g.wavemajor ? in[k * rowstride + si] : in[(int64_t)si * (M * M * HX) + k])
-                        : mk(T(0), T(0));
+    const int64_t kstride = g.wavemajor ? (int64_t)g.C * g.Kc : 1;
+    const cpx<T>* in = g.wavemajor ? spec + (int64_t)ch * g.Kc + S0 : spec + ((int64_t)ch * g.Kc + S0) * (M * MH);
+    for (int i = tid; i < NS * MH; i += BLK_THREADS) {
+      const int s = i % NS, j = i / NS;  // j = ky HX + kx, wavevector k = kz MH + j
+      const cpx<T>* c = in + (g.wavemajor ? (int64_t)s : (int64_t)s * (M * MH)) + j * kstride;
+      cpx<T> v[M];
+#pragma unroll
+      for (int n = 0; n < M; ++n) v[n] = s < ncell ? c[n * MH * kstride] : mk(T(0), T(0));
+      dft_reg<T, M, 1>(v);
+#pragma unroll
+      for (int u = 0; u < W; ++u) F[u * MH * NS + i] = v[(u - CR) & (M - 1)];
     }
   }
   __syncthreads();
-  // z pass: column (ky, kx, cell) -> kept rows uz < W
-  for (int col = tid; col < NCOL; col += nt) {
-    cpx<T> v[M];
-#pragma unroll
-    for (int j = 0; j < M; ++j) v[j] = F[bitrev(j, LB) * NCOL + col];
-    ifft_reg<T, M>(v, wp);
-#pragma unroll
-    for (int u = 0; u < W; ++u) F[u * NCOL + col] = v[(u - CR) & (M - 1)];
-  }
-  __syncthreads();
   // y pass: column (uz, kx, cell) over ky -> kept rows uy < W
-  constexpr int NY = NS * HX * W;
-  for (int yc = tid; yc < NY; yc += nt) {
-    const int kxs = yc % (HX * NS), uz = yc / (HX * NS);
-    cpx<T>* base = F + (size_t)uz * NCOL + kxs;
+  for (int i = tid; i < NS * HX * W; i += BLK_THREADS) {
+    const int kxs = i % (HX * NS), uz = i / (HX * NS);
+    cpx<T>* base = F + uz * MH * NS + kxs;
     cpx<T> v[M];
 #pragma unroll
-    for (int j = 0; j < M; ++j) v[j] = base[bitrev(j, LB) * HX * NS];
-    ifft_reg<T, M>(v, wp);
+    for (int n = 0; n < M; ++n) v[n] = base[n * HX * NS];
+    dft_reg<T, M, 1>(v);
 #pragma unroll
     for (int u = 0; u < W; ++u) base[u * HX * NS] = v[(u - CR) & (M - 1)];
   }
   __syncthreads();
-  // x pass (real output): row (uz, uy, cell): out[ux] = sum_kx w_kx Re(Y[kx] exp(+2 pi i kx t(ux) / M))
-  constexpr int NX = NS * W * W;
-  for (int xr = tid; xr < NX; xr += nt) {
-    const int si = xr % NS, uy = (xr / NS) % W, uz = xr / (NS * W);
-    const cpx<T>* Y = F + (size_t)uz * NCOL + (size_t)uy * HX * NS + si;
-    T out[W];
+  // x pass: row (uz, uy, cell) of Y[kx] = conj Y[M - kx] -> M reals x_t = sum_kx Y[kx] w^(kx t),
+  // w = exp(2 pi i / M): x_2n + i x_2n+1 is the M/2-point DFT of
+  // (Y[k] + conj Y[M/2-k]) + i w^k (Y[k] - conj Y[M/2-k])
+  for (int i = tid; i < NS * W * W; i += BLK_THREADS) {
+    const int s = i % NS, uy = (i / NS) % W, uz = i / (NS * W);
+    cpx<T>* Y = F + (uz * MH + uy * HX) * NS + s;
+    cpx<T> y[HX], z[M / 2];
 #pragma unroll
-    for (int u = 0; u < W; ++u) out[u] = T(0);
+    for (int k = 0; k < HX; ++k) y[k] = Y[k * NS];
+    y[0].y = T(0);  // real, as the half spectrum of a real signal
+    y[M / 2].y = T(0);
 #pragma unroll
-    for (int kx = 0; kx < HX; ++kx) {
-      const T wk = (kx == 0 || 2 * kx == M) ? T(1) : T(2);
-      const cpx<T> y = Y[kx * NS];
-      const T yr = wk * y.x, yi = wk * y.y;
-#pragma unroll
-      for (int u = 0; u < W; ++u) {
-        const cpx<T> w = wp[(kx * ((u - CR) & (M - 1))) & (M - 1)];
-        out[u] += yr * w.x - yi * w.y;
-      }
+    for (int k = 0; k < M / 2; ++k) {
+      const cpx<T> a = y[k], b = conjg(y[M / 2 - k]);
+      const cpx<T> d = rotate<T, M, 1>(a - b, k);
+      z[k] = mk(a.x + b.x - d.y, a.y + b.y + d.x);
     }
-    const int64_t S = S0 + si;
-    if (S < g.Kc) {
-      T* o = region + ((int64_t)ch * g.Kc + S) * W3 + ((size_t)uz * W + uy) * W;
+    dft_reg<T, M / 2, 1>(z);
 #pragma unroll
-      for (int u = 0; u < W; ++u) o[u] = out[u];
-    }
+    for (int q = 0; q < W / 2; ++q) Y[q * NS] = z[((2 * q - CR) & (M - 1)) / 2];
+  }
+  __syncthreads();
+  constexpr int WP = W / 2;
+  for (int i = tid; i < NS * (W3 / 2); i += BLK_THREADS) {
+    const int s = i % NS, q = i / NS, row = q / WP;
+    if (s >= ncell) continue;
+    const cpx<T> v = F[((row / W) * MH + (row % W) * HX + q % WP) * NS + s];
+    reinterpret_cast<cpx<T>*>(region + ((int64_t)ch * g.Kc + S0 + s) * W3)[q] = v;
   }
 }
 
-// Sum of the kept block outputs of the (2c+1)^3 coarse source cells around the
-// coarse cell T3 of fine cell (A3 within it), for the real channel ch.
-template <typename T>
-__device__ __forceinline__ T gather_kept(const T* __restrict__ region, const BlockGeo& g, int ch, const int* T3,
-                                         const int* A3, int periodic) {
+// Sums of the kept block outputs of the (2c+1)^3 coarse source cells around the
+// coarse cell T3 of fine cell (A3 within it), for the N real channels ch ... (past the
+// last one: zero).
+template <int N, typename T>
+__device__ __forceinline__ void gather_kept(const T* __restrict__ region, const BlockGeo& g, int ch, const int* T3,
+                                            const int* A3, int periodic, T* acc) {
   const int r = g.r, c = g.c, W = g.W, W3 = W * W * W;
-  const int64_t cb = (int64_t)ch * g.Kc;
-  T acc = T(0);
+#pragma unroll
+  for (int j = 0; j < N; ++j) acc[j] = T(0);
   for (int dz = -c; dz <= c; ++dz)
     for (int dy = -c; dy <= c; ++dy)
       for (int dx = -c; dx <= c; ++dx) {
@@ -524,18 +570,23 @@ __device__ __forceinline__ T gather_kept(const T* __restrict__ region, const Blo
         if (!ok) continue;
         const int64_t S = (int64_t)S3[0] + (int64_t)g.nc[0] * (S3[1] + (int64_t)g.nc[1] * S3[2]);
         const int u = (dx * r + A3[0] + c * r) + W * ((dy * r + A3[1] + c * r) + W * (dz * r + A3[2] + c * r));
-        acc += region[(cb + S) * W3 + u];
+        const T* q = region + ((int64_t)ch * g.Kc + S) * W3 + u;
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+          if (ch + j < g.C) acc[j] += q[(int64_t)j * g.Kc * W3];
       }
-  return acc;
 }
 
 // Fine locals through the child matrices: L'_f[co][t] = sum_ci Um[a][co][ci] L'_c[ci][T]
-// + the kept block outputs.  One thread per (fine cell, real output channel).
+// + the kept block outputs.  One thread per (fine cell, LM_CO real output channels): the
+// coarse local and the neighbour arithmetic are shared by the channels.
+// Bound by L1 requests (one per channel pair and thread before).
+constexpr int LM_CO = 4;
 template <typename T>
 __global__ void __launch_bounds__(128) local_matrix_kernel(const T* __restrict__ Lc, const T* __restrict__ region,
                                                            const T* __restrict__ Um, T* __restrict__ Lf, BlockGeo g,
                                                            int periodic) {
-  const int co = blockIdx.y;
+  const int co = blockIdx.y * LM_CO;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= g.Kf) return;
   const int r = g.r, C = g.C;
@@ -543,11 +594,38 @@ __global__ void __launch_bounds__(128) local_matrix_kernel(const T* __restrict__
   const int T3[3] = {tx / r, ty / r, tz / r}, A3[3] = {tx % r, ty % r, tz % r};
   const int64_t Tc = (int64_t)T3[0] + (int64_t)g.nc[0] * (T3[1] + (int64_t)g.nc[1] * T3[2]);
   const int a = A3[0] + r * (A3[1] + r * A3[2]);
-  const T* row = Um + ((int64_t)a * C + co) * C;
-  T acc = T(0);
-  for (int ci = 0; ci < C; ++ci) acc += __ldg(row + ci) * __ldg(Lc + (int64_t)ci * g.Kc + Tc);
-  acc += gather_kept<T>(region, g, co, T3, A3, periodic);
-  Lf[(int64_t)co * g.Kf + t] = acc;
+  const T* row[LM_CO];
+  T acc[LM_CO], kept[LM_CO];
+#pragma unroll
+  for (int j = 0; j < LM_CO; ++j) {
+    row[j] = Um + ((int64_t)a * C + min(co + j, C - 1)) * C;
+    acc[j] = T(0);
+  }
+  if (sizeof(T) == 4 && C % 4 == 0) {  // FP32 rows on 16-byte boundaries: four entries a load
+    for (int ci = 0; ci < C; ci += 4) {
+      T l[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) l[k] = __ldg(Lc + (int64_t)(ci + k) * g.Kc + Tc);
+#pragma unroll
+      for (int j = 0; j < LM_CO; ++j) {
+        const float4 u = __ldg(reinterpret_cast<const float4*>(row[j] + ci));
+        acc[j] += T(u.x) * l[0];
+        acc[j] += T(u.y) * l[1];
+        acc[j] += T(u.z) * l[2];
+        acc[j] += T(u.w) * l[3];
+      }
+    }
+  } else {
+    for (int ci = 0; ci < C; ++ci) {
+      const T l = __ldg(Lc + (int64_t)ci * g.Kc + Tc);
+#pragma unroll
+      for (int j = 0; j < LM_CO; ++j) acc[j] += __ldg(row[j] + ci) * l;
+    }
+  }
+  gather_kept<LM_CO>(region, g, co, T3, A3, periodic, kept);
+#pragma unroll
+  for (int j = 0; j < LM_CO; ++j)
+    if (co + j < C) Lf[(int64_t)(co + j) * g.Kf + t] = acc[j] + kept[j];
 }
 
 // Fine locals straight from the complex formula (child matrices too large): L2L
@@ -570,9 +648,13 @@ __global__ void __launch_bounds__(128) local_kernel(const T* __restrict__ Lc, co
   cpx<T> acc = mk(T(0), T(0));
   l2l_term<T>(l, m, p, r, [&](int ch) { return __ldg(Lc + (int64_t)ch * g.Kc + Tc); },
               [&](int ch) { return __ldg(R + ch); }, acc);
-  acc.x += gather_kept<T>(region, g, sidx(l, m), T3, A3, periodic);
-  Lf[(int64_t)sidx(l, m) * g.Kf + t] = acc.x;
-  if (m > 0) Lf[(int64_t)sidx(l, -m) * g.Kf + t] = acc.y + gather_kept<T>(region, g, sidx(l, -m), T3, A3, periodic);
+  T kept;
+  gather_kept<1>(region, g, sidx(l, m), T3, A3, periodic, &kept);
+  Lf[(int64_t)sidx(l, m) * g.Kf + t] = acc.x + kept;
+  if (m > 0) {
+    gather_kept<1>(region, g, sidx(l, -m), T3, A3, periodic, &kept);
+    Lf[(int64_t)sidx(l, -m) * g.Kf + t] = acc.y + kept;
+  }
 }
 
 template <typename T>
@@ -617,13 +699,13 @@ BlockGeo make_geo(const HierGeo& h, int C) {
 template <typename T, int M, int R>
 cudaError_t forward_ct_run(const BlockGeo& g, const void* Mf, void* spec, const void* tw, cudaStream_t s) {
   constexpr int NS = fwd_ns(M, R, sizeof(T)), HX = M / 2 + 1;
-  const size_t smem = sizeof(cpx<T>) * (M + NS * HX * R * R + NS * HX * M * R) + sizeof(T) * NS * R * R * R;
+  const size_t smem = sizeof(cpx<T>) * (M + NS * HX * M * R) + sizeof(T) * NS * R * R * R;
   if (smem > 200 * 1024) return cudaErrorNotSupported;
   cudaError_t e =
       cudaFuncSetAttribute(block_forward_ct_kernel<T, M, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   dim3 grid((unsigned)((g.Kc + NS - 1) / NS), (unsigned)g.C);
-  block_forward_ct_kernel<T, M, R><<<grid, 256, smem, s>>>((const T*)Mf, (cpx<T>*)spec, (const cpx<T>*)tw, g);
+  block_forward_ct_kernel<T, M, R><<<grid, BLK_THREADS, smem, s>>>((const T*)Mf, (cpx<T>*)spec, (const cpx<T>*)tw, g);
   return cudaGetLastError();
 }
 
@@ -663,16 +745,19 @@ cudaError_t inverse_reg_run(const BlockGeo& g, const void* spec, void* region, c
 }
 
 template <typename T, int M, int W, int CR>
-cudaError_t inverse_fft_run(const BlockGeo& g, const void* spec, void* region, const void* tw, cudaStream_t s) {
-  constexpr int NS = inv_ns(M, sizeof(T));
-  const size_t smem = sizeof(cpx<T>) * ((size_t)M + (size_t)NS * M * M * (M / 2 + 1));
-  if (smem > 200 * 1024) return cudaErrorNotSupported;
-  cudaError_t e = cudaFuncSetAttribute(block_inverse_fft_kernel<T, M, W, CR>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  dim3 grid((unsigned)((g.Kc + NS - 1) / NS), (unsigned)g.C);
-  block_inverse_fft_kernel<T, M, W, CR><<<grid, 256, smem, s>>>((const cpx<T>*)spec, (T*)region, (const cpx<T>*)tw, g);
-  return cudaGetLastError();
+cudaError_t inverse_fft_run(const BlockGeo& g, const void* spec, void* region, cudaStream_t s) {
+  constexpr int NS = inv_ns(M, W, sizeof(T));
+  constexpr size_t smem = inv_smem(M, W, sizeof(T), NS);
+  if constexpr (smem > kInvSmem) {
+    return cudaErrorNotSupported;
+  } else {
+    cudaError_t e = cudaFuncSetAttribute(block_inverse_fft_kernel<T, M, W, CR>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    dim3 grid((unsigned)((g.Kc + NS - 1) / NS), (unsigned)g.C);
+    block_inverse_fft_kernel<T, M, W, CR><<<grid, BLK_THREADS, smem, s>>>((const cpx<T>*)spec, (T*)region, g);
+    return cudaGetLastError();
+  }
 }
 
 template <typename T>
@@ -680,11 +765,11 @@ cudaError_t inverse_run(const HierGeo& h, int C, const void* spec, void* region,
   const BlockGeo g = make_geo(h, C);
   // (c, r) = (1, 2), (1, 4), (2, 2), (1, 8), (2, 4): FFT passes while a block's half spectrum fits
   cudaError_t e = cudaErrorNotSupported;
-  if (g.m == 8 && g.W == 6) e = inverse_fft_run<T, 8, 6, 2>(g, spec, region, tw, s);
-  if (g.m == 16 && g.W == 12) e = inverse_fft_run<T, 16, 12, 4>(g, spec, region, tw, s);
-  if (g.m == 16 && g.W == 10) e = inverse_fft_run<T, 16, 10, 4>(g, spec, region, tw, s);
-  if (g.m == 32 && g.W == 24) e = inverse_fft_run<T, 32, 24, 8>(g, spec, region, tw, s);
-  if (g.m == 32 && g.W == 20) e = inverse_fft_run<T, 32, 20, 8>(g, spec, region, tw, s);
+  if (g.m == 8 && g.W == 6) e = inverse_fft_run<T, 8, 6, 2>(g, spec, region, s);
+  if (g.m == 16 && g.W == 12) e = inverse_fft_run<T, 16, 12, 4>(g, spec, region, s);
+  if (g.m == 16 && g.W == 10) e = inverse_fft_run<T, 16, 10, 4>(g, spec, region, s);
+  if (g.m == 32 && g.W == 24) e = inverse_fft_run<T, 32, 24, 8>(g, spec, region, s);
+  if (g.m == 32 && g.W == 20) e = inverse_fft_run<T, 32, 20, 8>(g, spec, region, s);
   if (e != cudaErrorNotSupported) return e;
   // kept widths (2c+1) r with (2c+1)^2 r^2 <= 1024: registers per thread column
   switch (g.W) {
@@ -754,7 +839,7 @@ cudaError_t launch_hier_local(const HierGeo& h, int p, bool fp64, const void* Lc
                               const void* rtab, const void* um, void* Lf, int periodic, cudaStream_t s, int* nl) {
   const BlockGeo g = make_geo(h, nterms(p));
   if (um) {
-    dim3 grid((unsigned)((g.Kf + 127) / 128), (unsigned)g.C);
+    dim3 grid((unsigned)((g.Kf + 127) / 128), (unsigned)((g.C + LM_CO - 1) / LM_CO));
     if (fp64)
       local_matrix_kernel<double><<<grid, 128, 0, s>>>((const double*)Lc, (const double*)region, (const double*)um,
                                                        (double*)Lf, g, periodic);
