@@ -110,6 +110,80 @@ PMMM_HD void stockham_bf_any(int R, const cpx<T>* in, cpx<T>* out, int L, int Ns
 #if defined(__CUDACC__)
 namespace pmmm {
 
+// cos(2 pi j / 32), j = 0 ... 8, and from it exp(s 2 pi i j / N) for N = 2 ... 32
+// (j and N constants after unrolling).
+__host__ __device__ constexpr double cos32(int j) {
+  j &= 31;
+  if (j > 16) j = 32 - j;
+  const double q[9] = {1.0, 0.98078528040323044913, 0.92387953251128675613, 0.83146961230254523708,
+                       0.70710678118654752440, 0.55557023301960222474, 0.38268343236508977173,
+                       0.19509032201612826785, 0.0};
+  return j <= 8 ? q[j] : -q[16 - j];
+}
+template <typename T, int N, int SGN>
+__device__ __forceinline__ cpx<T> rotate(cpx<T> v, int j) {
+  const int k = (j * (32 / N)) & 31;
+  if (k == 0) return v;
+  if (k == 16) return mk(-v.x, -v.y);
+  if (k == 8) return SGN > 0 ? mk(-v.y, v.x) : mk(v.y, -v.x);
+  if (k == 24) return SGN > 0 ? mk(v.y, -v.x) : mk(-v.y, v.x);
+  const T c = (T)cos32(k), sn = (T)(SGN > 0 ? cos32(k + 24) : -cos32(k + 24));  // sin(t) = cos(t - pi/2)
+  return mk(v.x * c - v.y * sn, v.x * sn + v.y * c);
+}
+
+// DFT of length N = 2 ... 32 in registers, exp(SGN 2 pi i j k / N), natural order on
+// both sides, every twiddle a constant.
+template <typename T, int N, int SGN>
+__device__ __forceinline__ void dft_reg(cpx<T>* v) {
+  if constexpr (N == 2) {
+    dft2(v);
+  } else if constexpr (N == 4) {
+    dft4(v, SGN);
+  } else if constexpr (N == 8) {
+    dft8(v, SGN);
+  } else {
+    constexpr int A = 4, B = N / 4;  // n = B n1 + n2, k = k1 + A k2
+    cpx<T> t[A][B];
+#pragma unroll
+    for (int n2 = 0; n2 < B; ++n2) {
+      cpx<T> a[A];
+#pragma unroll
+      for (int n1 = 0; n1 < A; ++n1) a[n1] = v[B * n1 + n2];
+      dft4(a, SGN);
+#pragma unroll
+      for (int k1 = 0; k1 < A; ++k1) t[k1][n2] = rotate<T, N, SGN>(a[k1], n2 * k1);
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < A; ++k1) {
+      dft_reg<T, B, SGN>(t[k1]);
+#pragma unroll
+      for (int k2 = 0; k2 < B; ++k2) v[k1 + A * k2] = t[k1][k2];
+    }
+  }
+}
+
+// The L outputs of N = L or L / 2 inputs, the rest zero: out[2 q + t] is the q-th output
+// of the N-point DFT of in_e w_L^(te).
+template <typename T, int L, int N, int SGN>
+__device__ __forceinline__ void dft_pad(const cpx<T>* in, cpx<T>* out) {
+  static_assert(L == N || L == 2 * N, "padded by at most 2");
+  if constexpr (L == N) {
+#pragma unroll
+    for (int e = 0; e < N; ++e) out[e] = in[e];
+    dft_reg<T, L, SGN>(out);
+  } else {
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      cpx<T> u[N];
+#pragma unroll
+      for (int e = 0; e < N; ++e) u[e] = rotate<T, L, SGN>(in[e], t * e);
+      dft_reg<T, N, SGN>(u);
+#pragma unroll
+      for (int q = 0; q < N; ++q) out[2 * q + t] = u[q];
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------
 // The same Stockham stages with the length, the stage radices and the direction
 // known at compile time (lengths 8 ... 512), so that every index and twiddle

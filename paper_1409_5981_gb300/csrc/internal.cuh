@@ -215,6 +215,8 @@ cudaError_t launch_twiddles(bool fp64, int L, void* tw, cudaStream_t s);
 // One CTA per channel, whole 3-D transform in shared memory (fft_fused.cu): FP32,
 // transform lengths <= 32, the physical planes' half spectrum <= 200 KB.
 bool fft_fused_applies(bool fp64, const Dims& d);
+// Cubic meshes of 8, 16 or 32 cells an axis among them (compile-time kernels).
+bool fft_cube_applies(bool fp64, const Dims& d);
 cudaError_t launch_fft_fused_forward(const void* in, void* spec, const Dims& d, int C, const FftTw& tw, cudaStream_t s,
                                      int* nlaunch);
 cudaError_t launch_fft_fused_inverse(const void* spec, void* out, const Dims& d, int C, const FftTw& tw, cudaStream_t s,
