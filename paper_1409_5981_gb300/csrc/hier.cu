@@ -415,7 +415,8 @@ __global__ void __launch_bounds__(1024) block_inverse_reg_kernel(const cpx<T>* _
 constexpr size_t kInvSmem = 112 * 1024;  // two blocks per SM
 constexpr size_t inv_smem(int M, int W, int esz, int ns) { return (size_t)(2 * esz) * ns * W * M * (M / 2 + 1); }
 constexpr int inv_ns(int M, int W, int esz) {
-  // cells per block: the largest power of two <= 8 that fits
+  // cells per block: the largest power of two <= 8 that fits (at m = 16, inverse stage of the
+  // case above: 4 cells at four blocks per SM 473 us, 16 at one block 465 us, 8 at two 401 us)
   int ns = 8;
   while (ns > 1 && inv_smem(M, W, esz, ns) > kInvSmem) ns /= 2;
   return ns;
