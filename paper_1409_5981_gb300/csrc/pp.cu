@@ -776,12 +776,13 @@ __device__ __forceinline__ void pp_staged(const float4* __restrict__ sa, const f
   for (; j < npair; ++j) pp_pair_v<SELF>(sa[j], sb[j], tx, ty, tz, pot, gx, gy, gz);
 }
 
-// The near sums of 32 targets of one cell (lane = target): pot, g of pp_target_kernel.
+// Adds the near sums of 32 targets of one cell (lane = target): pot, g of pp_target_kernel.
+// mask_all (the same for all lanes): r = 0 adds zero in every cell, not in the own one alone.
 template <int CUT>
 __device__ __forceinline__ void pp_crowd_warp(const float4 xi, int sbase, int ix, int iy, int iz,
                                               const float4* __restrict__ S2, const uint32_t* __restrict__ pair_start,
-                                              const PPParams& pp, float4* sa, float4* sb, float2& pot, float2& gx,
-                                              float2& gy, float2& gz) {
+                                              const PPParams& pp, bool mask_all, float4* sa, float4* sb, float2& pot,
+                                              float2& gx, float2& gy, float2& gz) {
   const int lane = threadIdx.x & 31;
   for (int dz = -CUT; dz <= CUT; ++dz)
     for (int dy = -CUT; dy <= CUT; ++dy)
@@ -797,7 +798,7 @@ __device__ __forceinline__ void pp_crowd_warp(const float4 xi, int sbase, int ix
         const float ux = xi.x - (float)dx * pp.cs32[0], uy = xi.y - (float)dy * pp.cs32[1],
                     uz = xi.z - (float)dz * pp.cs32[2];
         const float2 tx = make_float2(ux, ux), ty = make_float2(uy, uy), tz = make_float2(uz, uz);
-        const bool own = dx == 0 && dy == 0 && dz == 0;
+        const bool mask = mask_all || (dx == 0 && dy == 0 && dz == 0);
         for (int p = pb; p < pe; p += 32) {
           const int m = min(32, pe - p);
           __syncwarp();
@@ -806,7 +807,7 @@ __device__ __forceinline__ void pp_crowd_warp(const float4 xi, int sbase, int ix
             sb[lane] = __ldg(S2 + 2 * (int64_t)(p + lane) + 1);
           }
           __syncwarp();
-          if (own)
+          if (mask)
             pp_staged<true>(sa, sb, m, tx, ty, tz, pot, gx, gy, gz);
           else
             pp_staged<false>(sa, sb, m, tx, ty, tz, pot, gx, gy, gz);
@@ -838,8 +839,16 @@ __global__ void __launch_bounds__(PPS_THREADS, 4) pp_target_kernel(
     if (crowd) {
       float2 pot = make_float2(0.f, 0.f), gx = pot, gy = pot, gz = pot;
       float4(*st)[32] = stage[threadIdx.x >> 5];
-      pp_crowd_warp<CUT>(xi, sbase, ix, iy, iz, reinterpret_cast<const float4*>(S2), pair_start, pp, st[0], st[1], pot,
-                         gx, gy, gz);
+      // r = 0 is looked for in the own cell only (a compare and a select per source).  A pair
+      // across a cell face can coincide too, after the rounding of its cell-relative
+      // coordinates; its infinite term leaves the sum of the potential infinite or NaN, and
+      // the warp then starts again with the test in every cell.
+      for (bool mask_all = false;; mask_all = true) {
+        pp_crowd_warp<CUT>(xi, sbase, ix, iy, iz, reinterpret_cast<const float4*>(S2), pair_start, pp, mask_all, st[0],
+                           st[1], pot, gx, gy, gz);
+        if (mask_all || __all_sync(0xffffffffu, isfinite(pot.x + pot.y))) break;
+        pot = gx = gy = gz = make_float2(0.f, 0.f);
+      }
       pa = pot.x; pbv = pot.y; xa = gx.x; xb = gx.y; ya = gy.x; yb = gy.y; za = gz.x; zb = gz.y;
     } else {
       f2 pot = pk2(0.f, 0.f), gx = pot, gy = pot, gz = pot;
