@@ -10,7 +10,8 @@
 // owning target l mod TL and source phase l / TL (TL = R rounded up to a power of two,
 // so a chunk of 8 targets still keeps 32 lanes busy on 4 source phases); sparse FP32
 // systems: one thread per target (pp_target_kernel); FP64: one block per item
-// (pp64_kernel).  Self pairs (r = 0) add zero.
+// (pp64_kernel).  Pairs at r = 0 (the self pair, and particles that coincide after the
+// rounding of their coordinates) add zero.
 #include "internal.cuh"
 #include "tcgen05.cuh"
 
@@ -410,10 +411,13 @@ __global__ void __launch_bounds__(PP_WARPS * 32, nt_blocks_per_sm<CUT>()) pp_ker
   const uint32_t nitems = item_start[K];
   const int nx = pp.n[0], ny = pp.n[1], nz = pp.n[2];
   const float csx = pp.cs32[0], csy = pp.cs32[1], csz = pp.cs32[2];
+  uint32_t item = 0;
+  bool again = false;  // the same item once more, r = 0 masked in every cell (below)
   for (;;) {
-    uint32_t item = 0;
-    if (lane == 0) item = atomicAdd(counter, 1u);  // one item per atomic: the shortest tail
-    item = __shfl_sync(0xffffffffu, item, 0);
+    if (!again) {
+      if (lane == 0) item = atomicAdd(counter, 1u);  // one item per atomic: the shortest tail
+      item = __shfl_sync(0xffffffffu, item, 0);
+    }
     if (item >= nitems) break;  // warp-uniform
     const int cell = (int)item_cell[item];
     const int chunk = (int)(item - item_start[cell]);
@@ -476,6 +480,7 @@ __global__ void __launch_bounds__(PP_WARPS * 32, nt_blocks_per_sm<CUT>()) pp_ker
     const int real_end = total;        // dummies of the tail: [real_end, total)
     total = (total + 3) & ~3;
     const int nch = (total + NT_CAP - 1) / NT_CAP;
+    const int nmask = again ? total : nselfp;  // pairs swept with r = 0 masked
     // queues the copies of chunk ch into buffer b (real pairs only)
     auto issue = [&](int ch, int b) {
       const int base = ch * NT_CAP, end = min(base + NT_CAP, total);
@@ -550,13 +555,18 @@ __global__ void __launch_bounds__(PP_WARPS * 32, nt_blocks_per_sm<CUT>()) pp_ker
       }
       __syncwarp();
       // own-cell pairs (self pair masked), then the rest of the chunk in one sweep
-      const int s1 = min(max(nselfp - base, 0), end - base);
+      const int s1 = min(max(nmask - base, 0), end - base);
       if (s1 > 0) pp_sweep<true>(buf, s1, ph, SP, tx, ty, tz, pot, gx, gy, gz);
       if (end - base > s1) pp_sweep<false>(buf + 2 * s1, end - base - s1, ph, SP, tx, ty, tz, pot, gx, gy, gz);
       __syncwarp();  // every lane is done with buffer b
       if (ch + 2 < nch) issue(ch + 2, b);
     }
     if (!__all_sync(0xffffffffu, ok)) return;
+    // r = 0 is masked in the own cell, which holds the self pair.  A pair across a cell face
+    // that coincides after the rounding of its coordinates leaves the potential's sum infinite
+    // or NaN; the item then runs a second time with every cell masked
+    again = !again && !__all_sync(0xffffffffu, !active || isfinite(pot.x + pot.y));
+    if (again) continue;
     float ps = pot.x + pot.y, gxs = -(gx.x + gx.y), gys = -(gy.x + gy.y), gzs = -(gz.x + gz.y);
     for (int o = TL; o < 32; o <<= 1) {
       ps += __shfl_xor_sync(0xffffffffu, ps, o);

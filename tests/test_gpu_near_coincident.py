@@ -75,3 +75,10 @@ def _check(pk, near, m, cutoff):
 @pytest.mark.parametrize("m", [3, 100])
 def test_per_target(pk, m, cutoff):
     _check(pk, pk.NEAR_PER_TARGET, m, cutoff)
+
+
+@pytest.mark.parametrize("cutoff", [1, 2])
+@pytest.mark.parametrize("m", [3, 100])
+@pytest.mark.parametrize("split", [False, True])
+def test_cell_items(pk, split, m, cutoff):
+    _check(pk, pk.NEAR_CELL_ITEMS_SPLIT if split else pk.NEAR_CELL_ITEMS, m, cutoff)
