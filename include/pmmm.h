@@ -266,10 +266,12 @@ enum {
  * whichever near-field kernel it takes): after the sort, the far field (P2M,
  * mesh stage, periodic corrections, L2P) runs on a second stream of the plan,
  * created with the highest priority, beside the near field, whose sums
- * go to a workspace buffer (16 bytes per particle, allocated on the first plain
- * call that needs it); one more launch adds the two.  The results equal those of
- * the one-stream sequence bit for bit.  One stream while stage timing is on, for
- * surrogate evaluations and inside a capture that would need the buffer first. */
+ * go to a workspace buffer (16 bytes per particle, at most 2 MB under
+ * PMMM_NEAR_AUTO, allocated with the particle workspace; after an autotuner's
+ * choice on its first call); one more launch adds the two.  The results equal
+ * those of the one-stream sequence bit for bit.  One stream while stage timing is
+ * on, for surrogate evaluations, inside a capture that would need the buffer
+ * first, and under PMMM_NEAR_AUTO when there was no memory for the buffer. */
 /* The M2L arithmetic that actually ran.  PMMM_FP32_SPLITBF16_M2L asks for the
  * tensor cores, but they serve only where the per-wavevector M2L is a true matrix
  * product: batched evaluations of more than one system, and the fine-level block

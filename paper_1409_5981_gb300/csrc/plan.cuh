@@ -117,12 +117,13 @@ struct pmmm_plan {
   size_t ws_bytes = 0;
   bool timing = false, timed = false;
   cudaEvent_t ev[ST_COUNT + 1] = {};
-  // split evaluation (PMMM_NEAR_CELL_ITEMS_SPLIT, FP32): the far field (P2M .. L2P)
-  // runs on `aux` beside the near field, which leaves its sums in `nearv` (float4
-  // per sorted particle); fork / join order the two streams
+  // split evaluation (FP32): the far field (P2M .. L2P) runs on `aux` beside the near
+  // field, which leaves its sums (float4 per sorted particle) in `nearv` where the
+  // schedule was chosen (PMMM_NEAR_CELL_ITEMS_SPLIT), in `nearv_auto` where the automatic
+  // one splits; fork / join order the two streams
   cudaStream_t aux = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-  void* nearv = nullptr;
+  void *nearv = nullptr, *nearv_auto = nullptr;
   bool split_last = false;
 };
 

@@ -67,6 +67,7 @@ void free_particles(pmmm_plan* pl) {
   dfree(pl, pl->epart);
   dfree(pl, pl->bpartial);
   dfree(pl, pl->nearv);
+  dfree(pl, pl->nearv_auto);
   pl->bchunks = 0;
   pl->max_items = 0;
   pl->cap = 0;
@@ -169,12 +170,11 @@ void set_streams(pmmm_plan* pl, cudaStream_t s);
 // cell 78 -> 62, 100 -> 68 us; 16^3, 5 / 32 per cell 110 -> 99, 154 -> 148 us; 32^3 p = 7,
 // 4 / 9 / 32 per cell 135 -> 134, 212 -> 213, 704 -> 716 us; 64^3 p = 5, 32: 4.83 -> 5.26 ms).
 constexpr int64_t SPLIT_AUTO_MAX = 1 << 17;
-// the near sums' buffer of the split evaluation is kept once a choice asks for it
-bool wants_split(const pmmm_plan* pl, int64_t cap) {
-  if (pl->fp64) return false;
-  return (pl->cfg.near_field == PMMM_NEAR_AUTO && cap <= 8 * SPLIT_AUTO_MAX) ||
-         pl->cfg.near_field == PMMM_NEAR_CELL_ITEMS_SPLIT || pl->tuned_near == PMMM_NEAR_CELL_ITEMS_SPLIT ||
-         pl->nearv != nullptr;
+// Buffers of the near sums: of a chosen split schedule for every particle, of the automatic
+// one for as many as it splits at most (2 MB), so that a reserved plan holds what later
+// calls need whatever their size.
+bool split_chosen(const pmmm_plan* pl) {
+  return (pl->tuned_near ? pl->tuned_near : pl->cfg.near_field) == PMMM_NEAR_CELL_ITEMS_SPLIT;
 }
 
 // Grows the mesh workspace to B systems (the particle workspace, sized by the
@@ -255,7 +255,11 @@ int ensure_particles(pmmm_plan* pl, int64_t n) {
   if (e == cudaSuccess) e = dalloc(pl, &v, sizeof(double) * 4 * (size_t)mi);
   if (e == cudaSuccess) pl->epart = (double*)v;
   if (e == cudaSuccess && !pl->fp64) e = dalloc(pl, &pl->src2, 32 * (size_t)pp_pairs_max(Kb, cap));
-  if (e == cudaSuccess && wants_split(pl, cap)) e = dalloc(pl, &pl->nearv, 16 * (size_t)cap);
+  if (e == cudaSuccess && !pl->fp64 && split_chosen(pl)) e = dalloc(pl, &pl->nearv, 16 * (size_t)cap);
+  // without this one the automatic schedule keeps one stream
+  if (e == cudaSuccess && !pl->fp64 && pl->cfg.near_field == PMMM_NEAR_AUTO &&
+      dalloc(pl, &pl->nearv_auto, 16 * (size_t)(cap < SPLIT_AUTO_MAX ? cap : SPLIT_AUTO_MAX)) != cudaSuccess)
+    cudaGetLastError();
   // items of one system: at most its cells + cap / 32 + 1
   const int bch = reduce_batched_chunks(pl->d.K, pp_items_max(pl->d.K, cap));
   if (e == cudaSuccess) e = dalloc(pl, &v, sizeof(double) * 5 * (size_t)pl->bcap * bch);
@@ -491,6 +495,7 @@ int run(pmmm_plan* pl, int B, int64_t n, const void* pos, const void* q, void* p
   const bool per_target = pp_per_target_applies(fp64, pl->g.c) &&
                           (near == PMMM_NEAR_PER_TARGET || (near == PMMM_NEAR_AUTO && sparse));
   bool split = false;
+  void* nearv = nullptr;  // buffer of the near sums (split evaluation)
   cudaStream_t fs = s;
   // energy partials and their reduction only for a call that returns the energy
   double* const epart = pl->want_energy ? pl->epart : nullptr;
@@ -521,19 +526,23 @@ int run(pmmm_plan* pl, int B, int64_t n, const void* pos, const void* q, void* p
   // and runs beside the near field, which then leaves its sums in nearv; a
   // combination launch follows both.  Not with stage timing (stages queued one
   // by one) nor with a far-field hook (the surrogate's own plans).
-  split = ((near == PMMM_NEAR_CELL_ITEMS_SPLIT && !per_target) || (near == PMMM_NEAR_AUTO && n <= SPLIT_AUTO_MAX)) &&
-          pl->aux && !pl->timing && !pl->hook && pl->src2;
-  if (split && !pl->nearv) {
-    // the near sums' buffer, allocated outside a capture (the plan's or the
-    // caller's; inside one the evaluation keeps one stream)
-    cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
-    const cudaError_t qe = pl->capturing ? cudaSuccess : cudaStreamIsCapturing(s, &cst);
-    if (qe != cudaSuccess) cudaGetLastError();  // only the answer matters here
-    if (pl->capturing || pl->cap <= 0 || qe != cudaSuccess || cst != cudaStreamCaptureStatusNone)
-      split = false;
-    else
-      CK(dalloc(pl, &pl->nearv, 16 * (size_t)pl->cap));
+  if (pl->aux && !pl->timing && !pl->hook && pl->src2) {
+    if (near == PMMM_NEAR_AUTO) {
+      if (n <= SPLIT_AUTO_MAX) nearv = pl->nearv_auto;
+    } else if (near == PMMM_NEAR_CELL_ITEMS_SPLIT && !per_target) {
+      if (!pl->nearv) {
+        // first call of a schedule that the autotuner chose: allocated outside a capture
+        // (the plan's or the caller's; inside one the evaluation keeps one stream)
+        cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
+        const cudaError_t qe = pl->capturing ? cudaSuccess : cudaStreamIsCapturing(s, &cst);
+        if (qe != cudaSuccess) cudaGetLastError();  // only the answer matters here
+        if (!pl->capturing && pl->cap > 0 && qe == cudaSuccess && cst == cudaStreamCaptureStatusNone)
+          CK(dalloc(pl, &pl->nearv, 16 * (size_t)pl->cap));
+      }
+      nearv = pl->nearv;
+    }
   }
+  split = nearv != nullptr;
   fs = s;
   if (split) {
     CK(cudaEventRecord(pl->ev_fork, s));
@@ -617,11 +626,11 @@ int run(pmmm_plan* pl, int B, int64_t n, const void* pos, const void* q, void* p
     const int64_t mi = pp_items_max(K, n);
     CK(launch_pp(fp64, pl->part, pl->src2, pl->pair_start, pl->vals_sorted, pl->keys_sorted, n, per_target, pl->cs, K,
                  pl->item_start, pl->item_cell, pl->counter, pl->num_sms, pl->far, pp, phi, force, epart, pl->err,
-                 split ? pl->nearv : nullptr, s, &nl));
+                 nearv, s, &nl));
     if (split) {
       CK(cudaStreamWaitEvent(s, pl->ev_join, 0));
       CK(launch_pp_combine(per_target, pl->part, pl->keys_sorted, pl->vals_sorted, n, pl->cs, K, pl->item_start,
-                           pl->item_cell, mi, pl->far, pl->nearv, pp, phi, force, epart, s, &nl));
+                           pl->item_cell, mi, pl->far, nearv, pp, phi, force, epart, s, &nl));
     }
     mark(pl, ST_REDUCE);
     if (!epart)
