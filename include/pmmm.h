@@ -262,16 +262,16 @@ enum {
   PMMM_INFO_SPLIT = 13      /* 1 if the last compute ran the far field beside the near field (below) */
 };
 /* Split evaluation (FP32 plans; near_field = PMMM_NEAR_CELL_ITEMS_SPLIT, set in the
- * config or chosen by pmmm_plan_autotune, and PMMM_NEAR_AUTO for small systems, with
- * whichever near-field kernel it takes): after the sort, the far field (P2M,
- * mesh stage, periodic corrections, L2P) runs on a second stream of the plan,
- * created with the highest priority, beside the near field, whose sums
- * go to a workspace buffer (16 bytes per particle, at most 2 MB under
- * PMMM_NEAR_AUTO, allocated with the particle workspace; after an autotuner's
- * choice on its first call); one more launch adds the two.  The results equal
- * those of the one-stream sequence bit for bit.  One stream while stage timing is
- * on, for surrogate evaluations, inside a capture that would need the buffer
- * first, and under PMMM_NEAR_AUTO when there was no memory for the buffer. */
+ * config or chosen by pmmm_plan_autotune; for small systems also PMMM_NEAR_AUTO, with
+ * whichever near-field kernel it takes, and the autotuner's per-target choice): after
+ * the sort, the far field (P2M, mesh stage, periodic corrections, L2P) runs on a second
+ * stream of the plan, created with the highest priority, beside the near field, whose
+ * sums go to a workspace buffer (16 bytes per particle, at most 2 MB under
+ * PMMM_NEAR_AUTO, allocated with the particle workspace; for an autotuner's choice by
+ * the autotuner or on its first call); one more launch adds the two.  The results equal
+ * those of the one-stream sequence bit for bit.  One stream while stage timing is on,
+ * for surrogate evaluations, inside a capture that would need the buffer first, and
+ * under PMMM_NEAR_AUTO when there was no memory for the buffer. */
 /* The M2L arithmetic that actually ran.  PMMM_FP32_SPLITBF16_M2L asks for the
  * tensor cores, but they serve only where the per-wavevector M2L is a true matrix
  * product: batched evaluations of more than one system, and the fine-level block
@@ -287,13 +287,15 @@ int pmmm_plan_info(pmmm_plan* plan, int what, int64_t* value);
 
 /* Autotuner: evaluates the given input (nsys systems; offsets as in
  * pmmm_compute_batched, or {0, n} for one system) once per candidate of each
- * tunable choice, timed over `reps` evaluations with CUDA events after one
- * warm-up, and keeps the fastest: the near-field schedule (cell items, cell items
- * with the far field beside them, or per target, where these apply) and, for
+ * tunable choice, timed over `reps` evaluations (graph launches for a single
+ * system, as its repeated calls) with CUDA events after a warm-up, and keeps the
+ * fastest: the near-field schedule (cell items or per
+ * target, each alone or with the far field beside it, where these apply) and, for
  * batched PMMM_FP32_SPLITBF16_M2L plans, the
  * systems per CTA of the tensor-core M2L (64 or 32).  The choice overrides the
  * config's near_field; results differ between choices only by the order of
- * floating-point sums.  Synchronous; reads back with PMMM_INFO_TUNED_NEAR and
+ * floating-point sums.  Synchronous; reads back with PMMM_INFO_TUNED_NEAR (per
+ * target in both forms: PMMM_INFO_SPLIT of the next compute tells them apart) and
  * PMMM_INFO_M2L_TILE. */
 int pmmm_plan_autotune(pmmm_plan* plan, int32_t nsys, const int64_t* offsets, const void* pos, const void* q,
                        int32_t reps);

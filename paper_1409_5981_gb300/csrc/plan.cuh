@@ -75,7 +75,7 @@ struct pmmm_plan {
     std::vector<int64_t> off;
     const void* ptr[4] = {nullptr, nullptr, nullptr, nullptr};
     uint64_t gen = 0;
-    int tune[2] = {0, 0};
+    int tune[3] = {0, 0, 0};
   };
   Graph graph[2];
   cudaStream_t cstream = nullptr;
@@ -90,6 +90,7 @@ struct pmmm_plan {
   const pmmm::FarHook* hook = nullptr;  // set by the surrogate for one evaluation
   // choices of pmmm_plan_autotune: near-field kernel (0: from the config), tensor-core M2L system tile
   int tuned_near = 0;
+  bool tuned_split = false;  // tuned_near is per target, with the far field beside it (small systems)
   int m2l_tile = 64;
   // two-level evaluation (cfg.refine >= 2): the coarse level runs on a one-level
   // plan of the coarse mesh; the block convolution of the fine level takes its

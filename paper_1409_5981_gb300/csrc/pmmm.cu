@@ -176,6 +176,12 @@ constexpr int64_t SPLIT_AUTO_MAX = 1 << 17;
 bool split_chosen(const pmmm_plan* pl) {
   return (pl->tuned_near ? pl->tuned_near : pl->cfg.near_field) == PMMM_NEAR_CELL_ITEMS_SPLIT;
 }
+// without this one the small evaluations keep one stream
+void alloc_nearv_auto(pmmm_plan* pl, int64_t cap) {
+  if (!pl->nearv_auto &&
+      dalloc(pl, &pl->nearv_auto, 16 * (size_t)(cap < SPLIT_AUTO_MAX ? cap : SPLIT_AUTO_MAX)) != cudaSuccess)
+    cudaGetLastError();
+}
 
 // Grows the mesh workspace to B systems (the particle workspace, sized by the
 // cell count, is rebuilt with it).
@@ -256,10 +262,8 @@ int ensure_particles(pmmm_plan* pl, int64_t n) {
   if (e == cudaSuccess) pl->epart = (double*)v;
   if (e == cudaSuccess && !pl->fp64) e = dalloc(pl, &pl->src2, 32 * (size_t)pp_pairs_max(Kb, cap));
   if (e == cudaSuccess && !pl->fp64 && split_chosen(pl)) e = dalloc(pl, &pl->nearv, 16 * (size_t)cap);
-  // without this one the automatic schedule keeps one stream
-  if (e == cudaSuccess && !pl->fp64 && pl->cfg.near_field == PMMM_NEAR_AUTO &&
-      dalloc(pl, &pl->nearv_auto, 16 * (size_t)(cap < SPLIT_AUTO_MAX ? cap : SPLIT_AUTO_MAX)) != cudaSuccess)
-    cudaGetLastError();
+  if (e == cudaSuccess && !pl->fp64 && (pl->cfg.near_field == PMMM_NEAR_AUTO || pl->tuned_split))
+    alloc_nearv_auto(pl, cap);
   // items of one system: at most its cells + cap / 32 + 1
   const int bch = reduce_batched_chunks(pl->d.K, pp_items_max(pl->d.K, cap));
   if (e == cudaSuccess) e = dalloc(pl, &v, sizeof(double) * 5 * (size_t)pl->bcap * bch);
@@ -527,7 +531,7 @@ int run(pmmm_plan* pl, int B, int64_t n, const void* pos, const void* q, void* p
   // combination launch follows both.  Not with stage timing (stages queued one
   // by one) nor with a far-field hook (the surrogate's own plans).
   if (pl->aux && !pl->timing && !pl->hook && pl->src2) {
-    if (near == PMMM_NEAR_AUTO) {
+    if (near == PMMM_NEAR_AUTO || (near == PMMM_NEAR_PER_TARGET && pl->tuned_split)) {
       if (n <= SPLIT_AUTO_MAX) nearv = pl->nearv_auto;
     } else if (near == PMMM_NEAR_CELL_ITEMS_SPLIT && !per_target) {
       if (!pl->nearv) {
@@ -749,7 +753,7 @@ int graph_eval(pmmm_plan* pl, int B, int64_t n, const int64_t* off, const void* 
   const bool same = g.exec && g.off.size() == (size_t)B + 1 &&
                     memcmp(g.off.data(), off, sizeof(int64_t) * (B + 1)) == 0 &&
                     memcmp(g.ptr, ptrs, sizeof(ptrs)) == 0 && g.gen == gen &&
-                    g.tune[0] == pl->tuned_near && g.tune[1] == pl->m2l_tile;
+                    g.tune[0] == pl->tuned_near && g.tune[1] == pl->m2l_tile && g.tune[2] == (int)pl->tuned_split;
   cudaError_t e = cudaSuccess;
   if (!same) {
     if (g.exec) cudaGraphExecDestroy(g.exec);
@@ -789,6 +793,7 @@ int graph_eval(pmmm_plan* pl, int B, int64_t n, const int64_t* off, const void* 
     g.gen = gen;
     g.tune[0] = pl->tuned_near;
     g.tune[1] = pl->m2l_tile;
+    g.tune[2] = pl->tuned_split;
   }
   e = cudaGraphLaunch(g.exec, pl->stream);
   if (e != cudaSuccess) return map_cuda(e);
@@ -1088,9 +1093,22 @@ int pmmm_plan_autotune(pmmm_plan* pl, int32_t nsys, const int64_t* offsets, cons
   }
   if (rc != PMMM_OK) return rc;
   if (n > 0 && (!pos || !q)) return PMMM_ERR_INVALID_ARG;
-  std::vector<int> nears = {pl->tuned_near};
-  if (pp_per_target_applies(pl->fp64, pl->g.c))
-    nears = {PMMM_NEAR_CELL_ITEMS, PMMM_NEAR_PER_TARGET, PMMM_NEAR_CELL_ITEMS_SPLIT};
+  // near-field kernel, and whether the per-target kernel has the far field beside it: the
+  // schedules that PMMM_NEAR_AUTO chooses among are all candidates
+  struct Schedule {
+    int near;
+    bool split;
+  };
+  std::vector<Schedule> nears = {{pl->tuned_near, pl->tuned_split}};
+  if (pp_per_target_applies(pl->fp64, pl->g.c)) {
+    nears = {{PMMM_NEAR_CELL_ITEMS, false}, {PMMM_NEAR_PER_TARGET, false}, {PMMM_NEAR_CELL_ITEMS_SPLIT, false}};
+    if (n <= SPLIT_AUTO_MAX) {
+      rc = ensure_particles(pl, n);
+      if (rc != PMMM_OK) return rc;
+      alloc_nearv_auto(pl, pl->cap);
+      nears.push_back({PMMM_NEAR_PER_TARGET, true});
+    }
+  }
   std::vector<int> tiles = {pl->m2l_tile};
   if (pl->m2l_tc && nsys > 1) tiles = {64, 32};
   cudaEvent_t e0, e1;
@@ -1103,15 +1121,26 @@ int pmmm_plan_autotune(pmmm_plan* pl, int32_t nsys, const int64_t* offsets, cons
   pl->timing = false;
   pl->want_energy = false;
   float best = 1e30f;
-  int best_near = pl->tuned_near, best_tile = pl->m2l_tile;
-  for (int nr : nears)
+  Schedule best_near = {pl->tuned_near, pl->tuned_split};
+  int best_tile = pl->m2l_tile;
+  for (const Schedule& nr : nears)
     for (int tl : tiles) {
-      pl->tuned_near = nr;
+      pl->tuned_near = nr.near;
+      pl->tuned_split = nr.split;
       pl->m2l_tile = tl;
+      // single systems as their repeated calls run, from a graph: the launch gaps of the plain
+      // sequence differ between the schedules (16^3 cells, c = 2, 4 particles a cell: plain
+      // 83 us per target beside the far field and 87 us split cell items, replayed 72 and 70)
+      const int64_t one[2] = {0, n};
+      auto eval = [&] {
+        return nsys == 1 ? graph_eval(pl, 1, n, one, pos, q, nullptr, nullptr)
+                         : run(pl, nsys, n, pos, q, nullptr, nullptr);
+      };
       rc = run(pl, nsys, n, pos, q, nullptr, nullptr);  // warm-up (allocates if needed)
+      if (rc == PMMM_OK) rc = eval();                   // captures
       cudaError_t ce = cudaSuccess;
       if (rc == PMMM_OK) ce = cudaEventRecord(e0, pl->stream);
-      for (int r = 0; r < reps && rc == PMMM_OK && ce == cudaSuccess; ++r) rc = run(pl, nsys, n, pos, q, nullptr, nullptr);
+      for (int r = 0; r < reps && rc == PMMM_OK && ce == cudaSuccess; ++r) rc = eval();
       if (rc == PMMM_OK && ce == cudaSuccess) ce = cudaEventRecord(e1, pl->stream);
       if (rc == PMMM_OK && ce == cudaSuccess) ce = cudaEventSynchronize(e1);
       float ms = 0.f;
@@ -1124,7 +1153,8 @@ int pmmm_plan_autotune(pmmm_plan* pl, int32_t nsys, const int64_t* offsets, cons
         best_tile = tl;
       }
     }
-  pl->tuned_near = best_near;
+  pl->tuned_near = best_near.near;
+  pl->tuned_split = best_near.split;
   pl->m2l_tile = best_tile;
   pl->timing = timing;
   cudaEventDestroy(e0);
