@@ -42,7 +42,7 @@ __device__ __forceinline__ float rsqrt_ftz(float x) {
 // from the upper word of x, about 20 bits) and one third-order Householder step,
 //   y = y0 + y0 e (1/2 + 3/8 e),  e = 1 - x y0^2,
 // whose remainder 5/16 e^3 is below 2^-58: five FP64 operations, at 64 cycles of an SM
-// quarter each.  Zero x gives 0, subnormal x the library's rsqrt(x).
+// quarter each.  Zero x gives 0, subnormal x the library's rsqrt(x); infinite x gives NaN.
 __device__ __forceinline__ double rsqrt64(double x) {
   double y0;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(P64_THREADS, P64_BLOCKS_PER_SM) pp64_kernel(
     if (active) {
       const int total = first[NN];
       int k = 0;
-      auto pair = [&](int e) {
+      auto pair = [&](int e, auto root) {
         while (e >= first[k + 1]) ++k;
         const double4 r = P[e + off[k]];
         const int ex = k % W, ey = (k / W) % W, ez = k / (W * W);
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(P64_THREADS, P64_BLOCKS_PER_SM) pp64_kernel(
           if (ez == d) uz = tz[d];
         }
         const double dx = ux - r.x, dy = uy - r.y, dz = uz - r.z;
-        const double ri = rsqrt64(fma(dx, dx, fma(dy, dy, dz * dz)));  // 0 for the self pair
+        const double ri = root(fma(dx, dx, fma(dy, dy, dz * dz)));  // 0 for the self pair
         const double qr = r.w * ri;
         pot += qr;
         const double qr3 = qr * (ri * ri);
@@ -161,10 +161,17 @@ __global__ void __launch_bounds__(P64_THREADS, P64_BLOCKS_PER_SM) pp64_kernel(
       };
       int e = ph;
       for (; e + NP < total; e += 2 * NP) {  // two at a time: 4.02 ms against 5.41 one by one (below)
-        pair(e);
-        pair(e + NP);
+        pair(e, rsqrt64);
+        pair(e + NP, rsqrt64);
       }
-      if (e < total) pair(e);
+      if (e < total) pair(e, rsqrt64);
+      // an infinite square (a particle flagged as far outside an open box), whose root is 0:
+      // the sums once more with the library's, one test per target instead of one per pair
+      if (isnan(pot)) {
+        pot = gx = gy = gz = 0.0;
+        k = 0;
+        for (e = ph; e < total; e += NP) pair(e, [](double x) { return x > 0.0 ? rsqrt(x) : 0.0; });
+      }
     }
     sum[0][tid] = pot;
     sum[1][tid] = gx;
