@@ -354,9 +354,10 @@ int64_t pp_pairs_max(int64_t K, int64_t n);
 // (epart[max_items][4]).  Persistent warps fetch items from *counter.  With
 // FP32, c = 1 and src2 given, the packed-FP32 kernel on the pair layout is used.
 // per_target (FP32, c = 1 only): one thread per sorted target (keys = sorted cell ids), for sparse cells.
-// near_out (split evaluation; FP32): the near sums of every
-// sorted target go to near_out[s] = (phi, grad) / (hs, hs^2) instead of being
-// combined, and launch_pp_combine adds the far field afterwards.
+// near_out (split evaluation; FP32): the near sums of every sorted target go to
+// near_out[s] instead of being combined, in the form that launch_pp_combine, which adds
+// the far field afterwards, takes for the same kernel (cell items: (phi, grad) in units
+// of 1 / hs and 1 / hs^2; per target: device units).
 bool pp_per_target_applies(bool fp64, int c);
 // epart may be null everywhere: no energy and force partials.
 cudaError_t launch_pp(bool fp64, const void* part, const void* src2, const uint32_t* pair_start, const uint32_t* vals,

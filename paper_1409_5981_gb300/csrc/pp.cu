@@ -686,8 +686,8 @@ __global__ void __launch_bounds__(256) pp_combine_kernel(const float4* __restric
 
 constexpr int PPS_THREADS = 256;
 
-// The end of a per-target evaluation for sorted target i (cell, near sums nr): adds the
-// far field, stores the results in the caller's order and reduces the energy and
+// The end of a per-target evaluation for sorted target i (cell, near sums nr in device
+// units): adds the far field, each sum in one rounding, stores the results in the caller's order and reduces the energy and
 // net-force terms per work item -- a segmented warp scan over lanes of equal item, one
 // store per item that lies inside the warp, and two double atomics (commutative, so
 // deterministic) on a zeroed slot for an item split between two warps.  Called by whole
@@ -711,8 +711,9 @@ __device__ __forceinline__ void target_epilogue(int64_t i, int64_t n, int cell, 
     te = min(tb + CHUNK, (int64_t)c1);
     const float4 fr = far[i];
     const float sg = pp.sign32, q = P[i].w;
-    const float pt = sg * (fr.x + nr.x);
-    const float g0 = sg * (fr.y + nr.y), g1 = sg * (fr.z + nr.z), g2 = sg * (fr.w + nr.w);
+    const float pt = sg * fmaf(nr.x, pp.ih32, fr.x);
+    const float g0 = sg * fmaf(nr.y, pp.ih2_32, fr.y), g1 = sg * fmaf(nr.z, pp.ih2_32, fr.z),
+                g2 = sg * fmaf(nr.w, pp.ih2_32, fr.w);
     const uint32_t o = vals[i];
     if (phi) phi[o] = pt;
     if (force) {
@@ -938,10 +939,7 @@ __global__ void __launch_bounds__(PPS_THREADS, 4) pp_target_kernel(
       up2(gy, ya, yb);
       up2(gz, za, zb);
     }
-    const float ps = pa + pbv, gxs = -(xa + xb), gys = -(ya + yb), gzs = -(za + zb);
-    // near sums in units of 1 / hs and 1 / hs^2, rounded on their own (as in pp_kernel_tma)
-    nr = make_float4(__fmul_rn(ps, pp.ih32), __fmul_rn(gxs, pp.ih2_32), __fmul_rn(gys, pp.ih2_32),
-                     __fmul_rn(gzs, pp.ih2_32));
+    nr = make_float4(pa + pbv, -(xa + xb), -(ya + yb), -(za + zb));
   }
   if (near_out) {  // split evaluation: the near sums only, combined later by pp_combine_target_kernel
     if (i < n) near_out[i] = nr;
