@@ -76,6 +76,9 @@ struct pmmm_plan {
     const void* ptr[4] = {nullptr, nullptr, nullptr, nullptr};
     uint64_t gen = 0;
     int tune[3] = {0, 0, 0};
+    int launches = 0;    // PMMM_INFO_LAUNCHES, _SPLIT and _M2L_ARITH of the captured evaluation
+    bool split = false;
+    int m2l_arith = -1;
   };
   Graph graph[2];
   cudaStream_t cstream = nullptr;

@@ -794,11 +794,17 @@ int graph_eval(pmmm_plan* pl, int B, int64_t n, const int64_t* off, const void* 
     g.tune[0] = pl->tuned_near;
     g.tune[1] = pl->m2l_tile;
     g.tune[2] = pl->tuned_split;
+    g.launches = pl->launches;
+    g.split = pl->split_last;
+    g.m2l_arith = pl->m2l_arith;
   }
   e = cudaGraphLaunch(g.exec, pl->stream);
   if (e != cudaSuccess) return map_cuda(e);
   pl->n_last = n;
   pl->nsys_last = B;
+  pl->launches = g.launches;
+  pl->split_last = g.split;
+  pl->m2l_arith = g.m2l_arith;
   return PMMM_OK;
 }
 
