@@ -6,10 +6,10 @@
 // GEMM: D[M x N] = A[M x K] . B[N x K]^T with A and B BF16 row-major (K
 // contiguous).  A CTA of 128 threads owns a 128 x TN tile (TN = 64, 128, 256):
 // K is staged 64 at a time into shared memory with 16-byte cp.async copies
-// (zero-filled past K or N) in the no-swizzle K-major core-matrix layout, two
-// stages deep; one thread issues the four K = 16 MMAs of a stage into the TMEM
-// accumulator and commits them to the stage's mbarrier, which frees the stage
-// for the copy two chunks ahead.  The epilogue reads the accumulator lane =
+// (zero-filled past K or N) in the no-swizzle K-major core-matrix layout, ST
+// stages deep (2 or 4); one thread issues the four K = 16 MMAs of a stage into the
+// TMEM accumulator and commits them to the stage's mbarrier, which frees the stage
+// for the copy ST chunks ahead.  The epilogue reads the accumulator lane =
 // row, 16 columns at a time, and applies bias, GELU or the GELU derivative.
 #include <cuda_bf16.h>
 
@@ -91,7 +91,23 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& a, int64_t m0, int n0,
   }
   for (int ch = 0; ch < nchunks; ++ch) {
     const int st = ch % ST;
-    cp_wait<ST - 2>();  // this thread's copies of chunk ch
+    const int nx = ch + ST - 1;  // goes into the stage that the MMAs of chunk ch - 1 read
+    auto refill = [&] {
+      if (nx < nchunks) {
+        if (ch >= 1 &&
+            !tc::bar_wait(tc::smem_u32(&bars[(ch - 1) % ST]), (uint32_t)(((ch - 1) / ST) & 1), G_WAIT_LIMIT))
+          ok = false;
+        load(nx);
+      }
+      cp_commit();
+    };
+    // this thread's copies of chunk ch; with two stages the next chunk's are queued first
+    if constexpr (ST == 2) {
+      refill();
+      cp_wait<1>();
+    } else {
+      cp_wait<ST - 2>();
+    }
     tc::fence_proxy_async();
     __syncthreads();
     if (tid == 0) {
@@ -103,14 +119,7 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& a, int64_t m0, int n0,
                      (ch | j) != 0);
       tc::commit(tc::smem_u32(&bars[st]));
     }
-    const int nx = ch + ST - 1;  // goes into the stage that the MMAs of chunk ch - 1 read
-    if (nx < nchunks) {
-      if (ch >= 1 &&
-          !tc::bar_wait(tc::smem_u32(&bars[(ch - 1) % ST]), (uint32_t)(((ch - 1) / ST) & 1), G_WAIT_LIMIT))
-        ok = false;
-      load(nx);
-    }
-    cp_commit();
+    if constexpr (ST > 2) refill();
   }
   const int last = nchunks - 1;
   const bool done = tc::bar_wait(tc::smem_u32(&bars[last % ST]), (uint32_t)((last / ST) & 1), G_WAIT_LIMIT);
@@ -472,8 +481,8 @@ unsigned grid_for(int64_t n, int threads, int64_t cap = 1 << 20) {
 }  // namespace
 
 namespace {
-constexpr int G_ST = 4;  // stages of the K pipeline
-size_t gemm_smem(int TN) { return G_ST * ((size_t)G_A_BYTES + (size_t)TN * G_KC * 2 + 8) + 16; }
+constexpr int G_ST = 4;  // stages of the K pipeline of small batches and of the weight gradients
+size_t gemm_smem(int TN, int ST) { return ST * ((size_t)G_A_BYTES + (size_t)TN * G_KC * 2 + 8) + 16; }
 bool gemm_ok(const GemmArgs& a) {
   if (a.M % 128 || a.N % 16 || a.K % 16 || a.K <= 0 || a.lda % 8 || a.ldb % 8) return false;
   return !((a.D32 && a.ldd % 4) || (a.D16 && a.ldd16 % 8) || (a.epi == GEMM_EPI_DGELU && (!a.Zin || a.ldz % 4)));
@@ -483,24 +492,30 @@ bool gemm_ok(const GemmArgs& a) {
 cudaError_t launch_gemm_tc(const GemmArgs& a, int num_sms, cudaStream_t s, int* nl) {
   if (a.M <= 0 || a.N <= 0) return cudaSuccess;
   if (!gemm_ok(a)) return cudaErrorInvalidValue;
-  // the widest tile that still gives two blocks per SM: latency (the K pipeline, then an
-  // epilogue of 40 instructions per element with GELU) is most of a block's time, so small
-  // batches want more and smaller blocks (8192 x 256 x 432 with GELU: 64 blocks of 256
-  // columns and two stages 31 us, 256 blocks of 64 columns and four stages 24 us, cold)
-  int TN = a.N > 128 ? 256 : (a.N > 64 ? 128 : 64);
-  while (TN > 64 && (int64_t)(a.M / 128) * ((a.N + TN - 1) / TN) < 2 * num_sms) TN /= 2;
+  // Large batches: whole rows of the output per block (A is read once) in two stages, so that
+  // two blocks of 256 columns fit an SM and one's epilogue runs beside the other's products.
+  // Small batches: latency (the K pipeline, then an epilogue of 40 instructions per element
+  // with GELU) is most of a block's time, so the narrowest tiles, for more blocks, and four
+  // stages.  A forward pass of 8192 rows 94 us in the first form, 72 in the second, 12288
+  // 96 and 98, 16384 97 and 108, 32768 155 and 184, 131072 446 and 516; the line lies at
+  // two thirds of a block per SM (13056 rows).
+  const int full = a.N > 128 ? 256 : (a.N > 64 ? 128 : 64);
+  const bool large = 3 * (int64_t)(a.M / 128) * ((a.N + full - 1) / full) >= 2 * (int64_t)num_sms;
+  const int TN = large ? full : 64;
   dim3 grid((unsigned)(a.M / 128), (unsigned)((a.N + TN - 1) / TN));
   cudaError_t e;
-#define GEMM_LAUNCH(T)                                                                                          \
-  e = cudaFuncSetAttribute(gemm_tc_kernel<T, G_ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(T)); \
-  if (e != cudaSuccess) return e;                                                                              \
-  gemm_tc_kernel<T, G_ST><<<grid, G_THREADS, gemm_smem(T), s>>>(a)
-  if (TN == 256) {
-    GEMM_LAUNCH(256);
+#define GEMM_LAUNCH(T, S)                                                                               \
+  e = cudaFuncSetAttribute(gemm_tc_kernel<T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(T, S)); \
+  if (e != cudaSuccess) return e;                                                                       \
+  gemm_tc_kernel<T, S><<<grid, G_THREADS, gemm_smem(T, S), s>>>(a)
+  if (!large) {
+    GEMM_LAUNCH(64, G_ST);
+  } else if (TN == 256) {
+    GEMM_LAUNCH(256, 2);
   } else if (TN == 128) {
-    GEMM_LAUNCH(128);
+    GEMM_LAUNCH(128, 2);
   } else {
-    GEMM_LAUNCH(64);
+    GEMM_LAUNCH(64, 2);
   }
 #undef GEMM_LAUNCH
   ++*nl;
@@ -543,9 +558,9 @@ cudaError_t launch_weight_grads(const GemmArgs g[3], const float* const dz[3], c
     ctot += cols[p];
   }
   cudaError_t e = cudaFuncSetAttribute(gemm_group_kernel<TN, G_ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)gemm_smem(TN));
+                                       (int)gemm_smem(TN, G_ST));
   if (e != cudaSuccess) return e;
-  gemm_group_kernel<TN, G_ST><<<dim3((unsigned)gg.tile0[G_GROUP], 1, (unsigned)used), G_THREADS, gemm_smem(TN), s>>>(gg);
+  gemm_group_kernel<TN, G_ST><<<dim3((unsigned)gg.tile0[G_GROUP], 1, (unsigned)used), G_THREADS, gemm_smem(TN, G_ST), s>>>(gg);
   const int rslice = (rows + slices - 1) / slices;
   colsum_kernel<<<dim3((unsigned)(ctot / 32), (unsigned)slices), 256, 0, s>>>(cs, rows, rslice, ctot, bpart);
   ss.wslices = used;
