@@ -67,6 +67,14 @@ __device__ __forceinline__ double rsqrt64(double x) {
 // FP64 issue rate).
 constexpr int P64_THREADS = 128;
 constexpr int P64_BLOCKS_PER_SM = 2;
+// Three blocks where there are many items of next to no pairs (the items are then a chain of
+// memory latencies): at least 2^14 particles, at most one to three cells.  60000 in 200
+// systems of 16^3 cells 3.65 -> 3.30 ms, 31457 / 64^3 uniform 2.77 -> 2.58 ms, in a Plummer
+// sphere 3.59 -> 3.82 ms: consecutive crowded items share an SM, which is why fuller cells
+// keep two (Plummer 8192 / 16^3 2.0 ms with two, 2.9 with three, 3.8 with four).
+inline int p64_blocks_per_sm(int64_t n, int64_t K) {
+  return n >= (1 << 14) && 3 * n <= K ? P64_BLOCKS_PER_SM + 1 : P64_BLOCKS_PER_SM;
+}
 
 template <int CUT>
 __global__ void __launch_bounds__(P64_THREADS, P64_BLOCKS_PER_SM) pp64_kernel(
@@ -998,7 +1006,7 @@ cudaError_t launch_pp(bool fp64, const void* part, const void* src2, const uint3
   if (fp64) {
     if (near_out) return cudaErrorInvalidValue;  // only the FP32 kernels split
 #define PP64(C)                                                                                                    \
-  pp64_kernel<C><<<(unsigned)(P64_BLOCKS_PER_SM * sms), P64_THREADS, 0, s>>>((const double*)part, vals, cell_start, K, \
+  pp64_kernel<C><<<(unsigned)(p64_blocks_per_sm(n, K) * sms), P64_THREADS, 0, s>>>((const double*)part, vals, cell_start, K, \
                                                                              item_start, item_cell, counter,       \
                                                                              (const double*)far, pp, (double*)phi, \
                                                                              (double*)force, epart)
