@@ -194,25 +194,31 @@ __global__ void __launch_bounds__(256) place_kernel(const uint32_t* __restrict__
   }
 }
 
-// Ranks of the RANK_THREADS indices that the block's threads hold among the indices
-// order[b .. e): the block sorts its own (bitonic, in shared memory), every index of
-// the range finds its place between them by bisection and is counted there, and a
-// running sum of the counts gives the ranks.  Returns the sorted index that the thread
-// takes on, its rank in *rank.  About 30 instructions per index and block, against
-// 2 RANK_THREADS for the plain comparison (2^20-particle Plummer sphere on 64^3 cells,
-// up to 6300 particles in a cell: sort stage 350 us with the plain comparison alone).
+// Ranks of the indices that the threads t0 .. of the block hold (the others pass NONE)
+// among the indices order[b .. e): the block sorts its own (bitonic, in shared memory),
+// every index of the range finds its place between them by bisection and is counted
+// there, and a running sum of the counts gives the ranks.  Returns the sorted index that
+// thread t0 + i takes on (the i-th), its rank in *rank.  About 30 instructions per index
+// and block, against 2 RANK_THREADS for the plain comparison (2^20-particle Plummer
+// sphere on 64^3 cells, up to 6300 particles in a cell: sort stage 350 us with the plain
+// comparison alone).
 constexpr int RANK_THREADS = 256;
 constexpr uint32_t RANK_CROWD = 1024;  // cells of at least this many particles
+constexpr uint32_t RANK_NONE = 0xffffffffu;
 
 __device__ __forceinline__ uint32_t crowded_rank(const uint32_t* __restrict__ order, uint32_t me, uint32_t b,
-                                                 uint32_t e, uint32_t* rank) {
+                                                 uint32_t e, int t0, uint32_t* rank) {
   __shared__ uint32_t srt[RANK_THREADS], cnt[RANK_THREADS + 1], wsum[RANK_THREADS / 32];
   const int t = threadIdx.x;
+  __syncthreads();  // the arrays may still be read from an earlier call
   srt[t] = me;
   cnt[t] = 0u;
   if (t == 0) cnt[RANK_THREADS] = 0u;
   __syncthreads();
+  // rolled loops: 32 registers, 56 otherwise, and the kernel is bound by loads in flight
+#pragma unroll 1
   for (int k = 2; k <= RANK_THREADS; k <<= 1)
+#pragma unroll 1
     for (int o = k >> 1; o > 0; o >>= 1) {
       const int p = t ^ o;
       if (p > t) {
@@ -224,6 +230,7 @@ __device__ __forceinline__ uint32_t crowded_rank(const uint32_t* __restrict__ or
       }
       __syncthreads();
     }
+#pragma unroll 2
   for (uint32_t i = b + t; i < e; i += RANK_THREADS) {
     const uint32_t v = order[i];
     int lo = 0;  // number of own indices <= v
@@ -243,8 +250,11 @@ __device__ __forceinline__ uint32_t crowded_rank(const uint32_t* __restrict__ or
   if ((t & 31) == 31) wsum[t >> 5] = x;
   __syncthreads();
   for (int w = 0; w < (t >> 5); ++w) x += wsum[w];
-  *rank = x;
-  return srt[t];
+  cnt[t] = x;  // only this thread's entry has been read so far
+  __syncthreads();
+  const int i = t >= t0 ? t - t0 : 0;
+  *rank = cnt[i];
+  return srt[i];
 }
 
 // The stable order, and with it everything an evaluation reads of a sorted particle:
@@ -269,18 +279,40 @@ __global__ void __launch_bounds__(RANK_THREADS) rank_gather_kernel(const uint32_
     for (int64_t i = (zero_all ? 0 : (int64_t)l.item_start[K]) + s; i < max_items;
          i += (int64_t)gridDim.x * blockDim.x)
       epart[i] = make_double4(0.0, 0.0, 0.0, 0.0);
-  if (n == 0) return;
+  if ((int64_t)blockIdx.x * RANK_THREADS >= n) return;  // the whole block
   const bool live = s < n;
   uint32_t me = order[live ? s : n - 1], c = keys[me], j = 0;
   const uint32_t b = (uint32_t)__ldg(l.cs + c), e = (uint32_t)__ldg(l.cs + c + 1);
-  // a block within one crowded cell sorts its 256 indices and counts the cell's others
-  // between them; otherwise every thread compares itself with all of its cell
-  __shared__ uint32_t first_cell;
-  if (threadIdx.x == 0) first_cell = c;
+  // The indices of a crowded cell are ranked by the block as a whole; such a cell is
+  // longer than a block, so it holds the block's first slot or its last.  Every other
+  // index is compared with all of its cell by its thread.  (Blocks that held parts of two
+  // cells compared all their indices so: sort stage of 786432 particles in a Plummer sphere
+  // on 32^3 cells 418 us, now 188; 163840 on 16^3 210 us, now 79.)
+  const bool crowd = live && e - b >= RANK_CROWD;
+  __shared__ uint32_t ends[2][3];  // cell, b, e
+  const int nlive = (int)min((int64_t)RANK_THREADS, n - (int64_t)blockIdx.x * RANK_THREADS);
+  if (threadIdx.x == 0 || (int)threadIdx.x == nlive - 1) {
+    uint32_t* q = ends[threadIdx.x == 0 ? 0 : 1];
+    q[0] = crowd ? c : RANK_NONE;
+    q[1] = b;
+    q[2] = e;
+    if (nlive == 1) ends[1][0] = RANK_NONE;  // one thread is both
+  }
   __syncthreads();
-  if (__syncthreads_and(live && c == first_cell && e - b >= RANK_CROWD)) {
-    me = crowded_rank(order, me, b, e, &j);
-  } else if (live) {
+#pragma unroll 1
+  for (int k = 0; k < 2; ++k) {
+    const uint32_t ck = ends[k][0];
+    if (ck == RANK_NONE || (k == 1 && ck == ends[0][0])) continue;
+    const int64_t s0 = (int64_t)ends[k][1] - (int64_t)blockIdx.x * RANK_THREADS;
+    uint32_t r;
+    const bool mine = live && c == ck;
+    const uint32_t v = crowded_rank(order, mine ? me : RANK_NONE, ends[k][1], ends[k][2], s0 > 0 ? (int)s0 : 0, &r);
+    if (mine) {
+      me = v;
+      j = r;
+    }
+  }
+  if (live && !crowd) {
     // whole 16-byte words; the entries outside [b, e) of the first and last are left out
     const uint4* o4 = reinterpret_cast<const uint4*>(order);
     uint32_t w = b / 4;
