@@ -712,7 +712,8 @@ cudaError_t inverse_fft_run(const BlockGeo& g, const void* spec, void* region, c
 template <typename T>
 cudaError_t inverse_run(const HierGeo& h, int C, const void* spec, void* region, const void* tw, cudaStream_t s) {
   const BlockGeo g = make_geo(h, C);
-  // (c, r) = (1, 2), (1, 4), (2, 2), (1, 8), (2, 4): FFT passes while a block's half spectrum fits
+  // (c, r) = (1, 2), (1, 4), (2, 2), (1, 8), (2, 4): register DFTs while a block's half spectra
+  // fit kInvSmem
   cudaError_t e = cudaErrorNotSupported;
   if (g.m == 8 && g.W == 6) e = inverse_fft_run<T, 8, 6, 2>(g, spec, region, s);
   if (g.m == 16 && g.W == 12) e = inverse_fft_run<T, 16, 12, 4>(g, spec, region, s);
@@ -720,14 +721,10 @@ cudaError_t inverse_run(const HierGeo& h, int C, const void* spec, void* region,
   if (g.m == 32 && g.W == 24) e = inverse_fft_run<T, 32, 24, 8>(g, spec, region, s);
   if (g.m == 32 && g.W == 20) e = inverse_fft_run<T, 32, 20, 8>(g, spec, region, s);
   if (e != cudaErrorNotSupported) return e;
-  // kept widths (2c+1) r with (2c+1)^2 r^2 <= 1024: registers per thread column
-  switch (g.W) {
-    case 6: return inverse_reg_run<T, 6>(g, spec, region, tw, s);
-    case 10: return inverse_reg_run<T, 10>(g, spec, region, tw, s);
-    case 12: return inverse_reg_run<T, 12>(g, spec, region, tw, s);
-    case 20: return inverse_reg_run<T, 20>(g, spec, region, tw, s);
-    case 24: return inverse_reg_run<T, 24>(g, spec, region, tw, s);
-    default: break;
+  // FP64 at m = 32, whose half spectra exceed that: registers per thread column
+  if constexpr (sizeof(T) == 8) {
+    if (g.W == 20) return inverse_reg_run<T, 20>(g, spec, region, tw, s);
+    if (g.W == 24) return inverse_reg_run<T, 24>(g, spec, region, tw, s);
   }
   const int NS = pick_ns<T>(g, true);
   const size_t smem = inverse_smem<T>(g, NS);
