@@ -46,18 +46,20 @@ typedef enum { PMMM_OPEN = 0, PMMM_PERIODIC = 1 } pmmm_boundary;
 
 /* Arithmetic of the hot path.  FP64: everything in double.  FP32: binning,
  * Green-function set-up and global reductions in double, P2M / FFT / M2L /
- * L2P / near field in float.  FP32_SPLITBF16_M2L is reserved for the batched
- * tensor-core M2L and currently behaves as FP32. */
+ * L2P / near field in float.  FP32_SPLITBF16_M2L: FP32 with the M2L of batched and
+ * two-level evaluations on the tensor cores (p <= 7; see PMMM_INFO_M2L_ARITH). */
 typedef enum { PMMM_FP64 = 0, PMMM_FP32 = 1, PMMM_FP32_SPLITBF16_M2L = 2 } pmmm_precision;
 
 /* Near-field kernel (Sec. 2.2's direct sum over the (2c+1)^3 nearest cells; the
  * choice changes only the order of floating-point sums):
  *   PMMM_NEAR_CELL_ITEMS  one warp per work item (a cell and up to 32 of its
  *                         particles), sources staged per warp: for filled cells
- *   PMMM_NEAR_PER_TARGET  one thread per particle (FP32 precisions, c = 1 only):
- *                         for sparsely filled cells
+ *   PMMM_NEAR_PER_TARGET  one thread per particle (FP32 precisions; FP64 plans run
+ *                         cell items): for sparsely filled cells
  *   PMMM_NEAR_AUTO        per target when N < PMMM_NEAR_AUTO_OCCUPANCY x cells
- *                         (and it applies), else cell items
+ *                         (and it applies), else cell items; FP32 evaluations of up to
+ *                         2^17 particles with the far field on a second stream beside
+ *                         either (see PMMM_INFO_SPLIT)
  *   PMMM_NEAR_CELL_ITEMS_SPLIT  cell items, with the far field on a second stream
  *                         beside them (FP32 precisions; see PMMM_INFO_SPLIT) */
 typedef enum {

@@ -1,4 +1,4 @@
-// Cell index along one axis, shared by the binning kernels (sort.cu, batch.cu).
+// Cell index along one axis, shared by the binning kernels (cellsort.cu, sort.cu).
 //
 // Cell index, in FP64 with every operation rounded (no contraction):
 //   t = x - lo;  if t is outside [0, len):

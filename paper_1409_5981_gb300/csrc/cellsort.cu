@@ -12,7 +12,8 @@
 //          decides, leaves no trace) and the sorted records in both layouts.
 // The rank launch compares each particle with all of its cell: as many comparisons as
 // the cell has pairs with itself, at 2 instructions each against 15 of the near field,
-// which takes those pairs and the ones with 26 or 124 more cells.
+// which takes those pairs and the ones with 26 or 124 more cells; cells of 1024 particles
+// or more are ranked by whole blocks instead (crowded_rank).
 // Latency-bound for small systems (4 dependent launches), bound by scattered 4- to
 // 16-byte accesses to the records for large ones.  Sort stage by CUDA events against
 // the radix sort it replaces (histogram, two scans and a scatter per 8-bit digit, cell

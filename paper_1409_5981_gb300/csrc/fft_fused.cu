@@ -9,10 +9,14 @@
 //            y pass in place; z pass from shared memory straight to the spectrum.
 //   inverse: z pass from the spectrum into shared memory (planes z < nz), y pass
 //            in place (rows y < ny kept), x pass to the real rows x < nx.
-// Every 1-D transform is held by one thread in registers: a radix-2
-// decimation-in-frequency FFT with all indices known at compile time, twiddles
-// broadcast from shared memory, output in bit-reversed order (reindexed at the
-// store).  Each channel is read and written once.
+// Every 1-D transform is held by one thread in registers; each channel is read and
+// written once.  Two families: runtime sizes (fft3_fwd_kernel, fft3_inv_kernel: radix-2
+// decimation-in-frequency FFTs, twiddles broadcast from shared memory, output in
+// bit-reversed order, reindexed at the store), for non-cubic meshes whose channels fill
+// the GPU; and cubes of 8, 16 or 32 cells with every size and twiddle a compile-time
+// constant (fft3_cube_fwd_kernel, fft3_cube_inv_kernel, below), for any number of
+// channels.  Only cubes, because the axis lengths of 4 to 32, padded or not, combine to
+// more than a hundred instances of each kernel.
 #include "fft.cuh"
 #include "internal.cuh"
 

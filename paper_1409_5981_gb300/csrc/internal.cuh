@@ -351,9 +351,9 @@ int64_t pp_items_max(int64_t K, int64_t n);
 int64_t pp_pairs_max(int64_t K, int64_t n);
 // Near field over the (2c+1)^3 cells plus the far field from `far`, written in
 // the caller's order to phi / force; energy and force partials per work item
-// (epart[max_items][4]).  Persistent warps fetch items from *counter.  With
-// FP32, c = 1 and src2 given, the packed-FP32 kernel on the pair layout is used.
-// per_target (FP32, c = 1 only): one thread per sorted target (keys = sorted cell ids), for sparse cells.
+// (epart[max_items][4]).  Persistent warps (FP32) or blocks (FP64) fetch items from
+// *counter; the FP32 kernels read the sources from the pair layout src2.
+// per_target (FP32): one thread per sorted target (keys = sorted cell ids), for sparse cells.
 // near_out (split evaluation; FP32): the near sums of every sorted target go to
 // near_out[s] instead of being combined, in the form that launch_pp_combine, which adds
 // the far field afterwards, takes for the same kernel (cell items: (phi, grad) in units

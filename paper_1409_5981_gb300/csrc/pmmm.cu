@@ -167,8 +167,9 @@ void set_streams(pmmm_plan* pl, cudaStream_t s);
 // The automatic near field splits evaluations of at most this many particles: there the
 // far field is a chain of launches that leave the GPU mostly idle, and the near field fits
 // beside it (graph-launched evaluations, one stream -> split: 8^3 cells p = 5, 9 / 32 per
-// cell 78 -> 62, 100 -> 68 us; 16^3, 5 / 32 per cell 110 -> 99, 154 -> 148 us; 32^3 p = 7,
-// 4 / 9 / 32 per cell 135 -> 134, 212 -> 213, 704 -> 716 us; 64^3 p = 5, 32: 4.83 -> 5.26 ms).
+// cell 52 -> 43, 81 -> 60 us; 16^3, 5 / 14 per cell 62 -> 49, 76 -> 69 us; 32^3 p = 7, 3 per
+// cell 105 -> 99 us; above the line, with the kernels of the time, 9 / 32 per cell
+// 212 -> 213, 704 -> 716 us; 64^3 p = 5, 32: 4.83 -> 5.26 ms).
 constexpr int64_t SPLIT_AUTO_MAX = 1 << 17;
 // Buffers of the near sums: of a chosen split schedule for every particle, of the automatic
 // one for as many as it splits at most (2 MB), so that a reserved plan holds what later

@@ -63,8 +63,8 @@ __device__ __forceinline__ double rsqrt64(double x) {
 // item's results depend only on the item.
 // Against one warp per item with power-of-two lane splits, per-cell loops and rsqrt():
 // 4096 particles / 8^3 open 303 -> 53 us (512 items over 608 SM quarters: a quarter of
-// them idle, others with three), 131072 / 16^3 periodic 4.83 -> 4.02 ms (86 % of the
-// FP64 issue rate).
+// them idle, others with three), 131072 / 16^3 periodic 4.83 -> 4.02 ms (81 % of the
+// FP64 issue rate in the pairs' 18 operations).
 constexpr int P64_THREADS = 128;
 constexpr int P64_BLOCKS_PER_SM = 2;
 // Three blocks where there are many items of next to no pairs (the items are then a chain of
@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(P64_THREADS, P64_BLOCKS_PER_SM) pp64_kernel(
         gz = fma(-qr3, dz, gz);
       };
       int e = ph;
-      for (; e + NP < total; e += 2 * NP) {  // two at a time: 4.02 ms against 5.41 one by one (below)
+      for (; e + NP < total; e += 2 * NP) {  // two at a time: 4.02 ms against 5.41 one by one
         pair(e, rsqrt64);
         pair(e + NP, rsqrt64);
       }
@@ -294,8 +294,7 @@ __device__ __forceinline__ void pp_pair2_mixed(const ulonglong2& A, const ulongl
 
 // FP32 near field (c = 1 or 2) with the neighbour cells staged by the Tensor Memory
 // Accelerator's bulk copies (cp.async.bulk, global -> shared, completion counted in
-// bytes on an mbarrier).  Same work items, lane mapping, results and energy
-// partials as the other cell-item kernels.  Per item the warp lists its (2c+1)^3 neighbour
+// bytes on an mbarrier).  Per item the warp lists its (2c+1)^3 neighbour
 // cells -- the target's own cell first, then the others in (z, y, x) order --
 // numbers their source pairs consecutively and streams them through two
 // shared-memory buffers of NT_CAP pairs: a buffer is filled by one bulk copy per
