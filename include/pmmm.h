@@ -68,7 +68,7 @@ typedef enum {
   PMMM_NEAR_PER_TARGET = 2,
   PMMM_NEAR_CELL_ITEMS_SPLIT = 3
 } pmmm_near_field;
-#define PMMM_NEAR_AUTO_OCCUPANCY 16
+#define PMMM_NEAR_AUTO_OCCUPANCY 8
 
 enum {
   PMMM_OK = 0,

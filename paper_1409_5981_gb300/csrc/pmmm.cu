@@ -490,11 +490,14 @@ int run(pmmm_plan* pl, int B, int64_t n, const void* pos, const void* q, void* p
   const bool fp64 = pl->fp64;
   const int64_t Ks = pl->d.K, K = Ks * B;  // cells per system, cells of all systems
   // near field: one thread per target when asked, or (automatic) when the cells
-  // hold fewer than PMMM_NEAR_AUTO_OCCUPANCY particles on average: the two kernels
-  // take the same time on uniform systems of 16 to 17 (c = 1) and 16 (c = 2) particles
-  // per cell (2^15 cells, c = 1: 12 per cell 133 us per target, 164 us items; 16: 209
-  // and 219 us; 24: 416 and 358 us).  Crowded cells of an uneven system cost the
-  // per-target kernel 1.2 times the items' time, no more
+  // hold fewer than PMMM_NEAR_AUTO_OCCUPANCY particles on average.  On uniform systems
+  // of 2^15 cells (whole evaluations, p = 5) the per-target kernel and the items take the
+  // same time at 10 (c = 1) and 9 (c = 2) particles per cell: c = 1, 4 per cell 98 and
+  // 126 us, 8: 146 and 160, 10: 182 and 182, 12: 220 and 212; c = 2, 8: 380 and 395, 10:
+  // 533 and 497.  Crowded cells make the per-target kernel slower by up to 1.7 times, its
+  // blocks of 256 consecutive targets being all crowded or all sparse (Plummer spheres on
+  // 2^15 cells, 8 per cell: c = 1 8.8 and 7.0 ms, c = 2 21.6 and 15.7 ms), hence the line
+  // at the lower end
   const bool sparse = n < (int64_t)PMMM_NEAR_AUTO_OCCUPANCY * K;
   const int near = pl->tuned_near ? pl->tuned_near : pl->cfg.near_field;
   const bool per_target = pp_per_target_applies(fp64, pl->g.c) &&
