@@ -494,21 +494,24 @@ cudaError_t launch_gemm_tc(const GemmArgs& a, int num_sms, cudaStream_t s, int* 
   if (!gemm_ok(a)) return cudaErrorInvalidValue;
   // Large batches: whole rows of the output per block (A is read once) in two stages, so that
   // two blocks of 256 columns fit an SM and one's epilogue runs beside the other's products.
-  // Small batches: latency (the K pipeline, then an epilogue of 40 instructions per element
-  // with GELU) is most of a block's time, so the narrowest tiles, for more blocks, and four
-  // stages.  A forward pass of 8192 rows 94 us in the first form, 72 in the second, 12288
-  // 96 and 98, 16384 97 and 108, 32768 155 and 184, 131072 446 and 516; the line lies at
-  // two thirds of a block per SM (13056 rows).
+  // Medium ones: 128 columns in two stages, three blocks per SM.  Small ones: latency (the K
+  // pipeline, then an epilogue of 40 instructions per element with GELU) is most of a block's
+  // time, so the narrowest tiles, for more blocks, and four stages.  Forward pass / training
+  // step in the three forms, us: 8192 rows 94 / 283, 73 / 236, 72 / 224; 12288 96 / 328, 91 / 305,
+  // 98 / 322; 16384 97 / 366, 97 / 348, 108 / 364; 24576 136 / 516, 133 / 480, 147 / 515; 32768 155 / 605, 178 / 658, 184 / 653; 131072
+  // 446 / 2020, 473 / 2005, 578 / 2232.  The lines lie at 0.6 (11776 rows) and 1.5 (29184 rows)
+  // blocks of whole rows per SM.
   const int full = a.N > 128 ? 256 : (a.N > 64 ? 128 : 64);
-  const bool large = 3 * (int64_t)(a.M / 128) * ((a.N + full - 1) / full) >= 2 * (int64_t)num_sms;
-  const int TN = large ? full : 64;
+  const int64_t blocks = (int64_t)(a.M / 128) * ((a.N + full - 1) / full);
+  const bool small = 5 * blocks < 3 * (int64_t)num_sms;
+  const int TN = small ? 64 : (2 * blocks < 3 * (int64_t)num_sms ? std::min(full, 128) : full);
   dim3 grid((unsigned)(a.M / 128), (unsigned)((a.N + TN - 1) / TN));
   cudaError_t e;
 #define GEMM_LAUNCH(T, S)                                                                               \
   e = cudaFuncSetAttribute(gemm_tc_kernel<T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(T, S)); \
   if (e != cudaSuccess) return e;                                                                       \
   gemm_tc_kernel<T, S><<<grid, G_THREADS, gemm_smem(T, S), s>>>(a)
-  if (!large) {
+  if (small) {
     GEMM_LAUNCH(64, G_ST);
   } else if (TN == 256) {
     GEMM_LAUNCH(256, 2);
