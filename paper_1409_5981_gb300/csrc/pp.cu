@@ -174,8 +174,9 @@ __global__ void __launch_bounds__(P64_THREADS, P64_BLOCKS_PER_SM) pp64_kernel(
       }
       if (e < total) pair(e, rsqrt64);
       // an infinite square (a particle flagged as far outside an open box), whose root is 0:
-      // the sums once more with the library's, one test per target instead of one per pair
-      if (isnan(pot)) {
+      // the sums once more with the library's, one test per target instead of one per pair (on
+      // the exponent, an integer operation)
+      if ((__double2hiint(pot) & 0x7ff00000) == 0x7ff00000) {
         pot = gx = gy = gz = 0.0;
         k = 0;
         for (e = ph; e < total; e += NP) pair(e, [](double x) { return x > 0.0 ? rsqrt(x) : 0.0; });
